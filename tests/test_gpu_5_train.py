@@ -105,6 +105,39 @@ def test_router_backward(A, shape, B, T, K):
     H.assert_close(H.to_np(yg), refg, H.tol(shape), "gated layer")
 
 
+@pytest.mark.parametrize("n,d,h,dtype,shift", [(1, 64, 64, "bf16", 0), (15, 192, 40, "f32", 1), (17, 4096, 64, "bf16", 0),
+                                              (263, 2048, 64, "f32", 0), (1000, 320, 64, "bf16", 1),
+                                              (33, 64, 3, "f32", 0)])
+def test_router_backward_edges(A, n, d, h, dtype, shift):
+    """Kept counts around the 16-row blocks and the eighths of the reduction,
+    feature widths that are not multiples of its 64 columns times the warps,
+    few hidden units, kept rows in any order, and an upstream gradient at an
+    odd float. Same inputs on both sides, so only fp32 sums differ: about
+    sqrt(d) + sqrt(n) roundings of 2^-24 each (under 1e-5 of the largest
+    element at these sizes)."""
+    shape = S.PYTHIA_70M.replace(d=d, router_hidden=h, n_layers=1, dtype=dtype)
+    td = H.tdtype(shape)
+    W = H.host_layer(shape, n + d)
+    BT = n + 37
+    x = S.round_to(S.hidden(n, 1, BT, d), dtype)
+    y = S.round_to(x + 0.3 * S.hidden(n + 1, 1, BT, d), dtype)
+    g = np.random.default_rng(n * d)
+    G = g.standard_normal((BT, d)).astype(np.float32)
+    rows = g.permutation(BT)[:n].astype(np.int32)
+    store = torch.empty(BT * d + 4, dtype=torch.float32, device="cuda")
+    Gd = store[shift:shift + BT * d].view(BT, d)
+    Gd.copy_(torch.from_numpy(G))
+    got = A.adadsf_router_backward(A.make_cfg(shape, A.FLAG_GATE_SIGMOID), A.to_device(W, td), H.to_dev(x, td),
+                                   H.to_dev(y, td), torch.from_numpy(rows).cuda(), Gd).cpu().numpy().astype(np.float64)
+    x64 = x.astype(np.float64)
+    delta = (y.astype(np.float64) - x64).reshape(BT, d)[rows]
+    ref = O.router_grad(x64, H.f64(W), rows, delta, G.astype(np.float64)[rows])
+    parts = {"router_w1": got[:h * d].reshape(h, d), "router_b1": got[h * d:h * d + h],
+             "router_w2": got[h * d + h:h * d + 2 * h], "router_b2": got[h * d + 2 * h:]}
+    for k, v in parts.items():
+        H.assert_close(v, ref[k], 2e-5, k)
+
+
 @pytest.mark.parametrize("shape,lr", [(S.PYTHIA_70M.replace(n_layers=1), 3000.0),
                                       (QWEN_SMALL.replace(dtype="f32"), 3000.0)])
 def test_router_alignment_descends(A, shape, lr):
