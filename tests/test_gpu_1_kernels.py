@@ -146,6 +146,24 @@ def test_linear_f32(A, M, N, Kd):
     assert H.max_rel(H.to_np(out), O.linear(x, w, None, "gelu")) < 1e-5
 
 
+@pytest.mark.parametrize("M,N,Kd,act", [(1, 4, 4, 0), (63, 36, 100, 1), (65, 516, 2052, 0), (129, 68, 64, 1),
+                                        (64, 512, 2048, 0), (700, 2048, 96, 1), (1532, 512, 2048, 0), (3001, 260, 36, 1)])
+def test_linear_f32_splits(A, M, N, Kd, act):
+    """Rows, columns and k around the edges of both fp32 tiles (64 x 32 and
+    128 x 64, 32 k a stage) and every cluster split of k. Error of an fp32 sum
+    of K random products against its result: under sqrt(K) 2^-24 of its rms, and
+    under 10 of that on the largest of 10^6 elements (3e-5 at K = 2052)."""
+    g = np.random.default_rng(M * N + Kd)
+    x = g.standard_normal((M, Kd)).astype(np.float32)
+    w = (0.05 * g.standard_normal((N, Kd))).astype(np.float32)
+    b = g.standard_normal(N).astype(np.float32)
+    out = torch.full((M + 1, N), 7.0, device="cuda")
+    A.adadsf_linear(H.to_dev(x, torch.float32), H.to_dev(w, torch.float32), H.to_dev(b, torch.float32), out[:M], act=act)
+    ref = O.linear(x, w, b.astype(np.float64), "gelu" if act else None)
+    H.assert_close(out[:M].cpu().numpy(), ref, 3e-5, "linear f32")
+    assert bool((out[M] == 7.0).all())          # nothing past the last row
+
+
 # ---------------------------------------------------------------- router (Sec. 3.4)
 @pytest.mark.parametrize("shape,n", [(S.PYTHIA_160M, 1), (S.PYTHIA_160M, 2048), (S.QWEN25_1_5B, 333),
                                      (S.PYTHIA_70M, 128), (S.PYTHIA_160M, 777), (S.PYTHIA_1_4B, 16384)])
