@@ -8,8 +8,11 @@
 // (a row of 512 fp32 features is 4 pieces a warp), transpose their pieces of x
 // and W1 into shared memory of their own (no block barrier in the loop, the
 // next piece already in flight in registers), and hold 4 rows x 8 units per
-// thread: three 16-byte shared loads feed 32 multiply-adds. The warps' partial
-// tiles are then added in warp order (bit-reproducible).
+// thread: three 16-byte shared loads feed 32 multiply-adds. Four lanes load a
+// row's piece (8 lines an instruction; a row per lane made 32 and kept the L1
+// pipe at 80 %), and the columns of the transposed pieces are XOR-ed with 8
+// times the loading lane's vector so that these stores spread over the banks.
+// The warps' partial tiles are then added in warp order (bit-reproducible).
 #pragma once
 
 #include "common.cuh"
@@ -31,35 +34,35 @@ struct RouterRows {
 };
 
 // u[row][unit] (no bias) of 4 consecutive units: thread t holds row t / 16 and
-// units u0 + 4 (t % 16) ... + 3 (zero past h). xr: row (lane % 16) of the tile
-// (any valid row for the ones past the end); w1 [h][d]; d a multiple of 64,
-// rows 16-byte aligned. Block-wide: shared memory is reused, with barriers
+// units u0 + 4 (t % 16) ... + 3 (zero past h). xr0, xr1: rows lane / 4 and lane / 4
+// + 8 of the tile (any valid row for the ones past the end); w1 [h][d]; d a
+// multiple of 64, rows 16-byte aligned. Block-wide: shared memory is reused, with barriers
 // on both sides.
 template <typename T>
-__device__ __forceinline__ float4 router_rows_units(const T* xr, const T* w1, int u0, int h, int d, float* smem) {
+__device__ __forceinline__ float4 router_rows_units(const T* xr0, const T* xr1, const T* w1, int u0, int h, int d, float* smem) {
   using R = RouterRows<T>;
   constexpr int V = Elem<T>::kVec, KC = R::KC;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float* ws = smem + warp * R::WARP_FLOATS;   // [KC][64]
   float* xs = ws + KC * kRrUnits;             // [KC][16]
   const int rg = lane >> 3, ug = lane & 7;
-  float acc[4][8];
+  float tot[4][8];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+    for (int j = 0; j < 8; ++j) tot[i][j] = 0.f;
   const int n = d / KC;
   uint4 wv[8], xv[2];
+  const int lrow = lane >> 2, lvec = lane & 3;
   auto fetch = [&](int c) {
-    const T* wp = w1 + (int64_t)c * KC;
+    const int64_t k = (int64_t)c * KC + lvec * V;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const int unit = u0 + lane + 32 * (i & 1);
-      wv[i] = unit < h ? *reinterpret_cast<const uint4*>(wp + (int64_t)unit * d + (i >> 1) * V) : make_uint4(0, 0, 0, 0);
+      const int unit = u0 + lrow + 8 * i;
+      wv[i] = unit < h ? *reinterpret_cast<const uint4*>(w1 + (int64_t)unit * d + k) : make_uint4(0, 0, 0, 0);
     }
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-      xv[i] = *reinterpret_cast<const uint4*>(xr + (int64_t)c * KC + ((lane >> 4) + 2 * i) * V);
+    xv[0] = *reinterpret_cast<const uint4*>(xr0 + k);
+    xv[1] = *reinterpret_cast<const uint4*>(xr1 + k);
   };
   if (warp < n) fetch(warp);
   for (int c = warp; c < n; c += kRrWarps) {
@@ -69,22 +72,28 @@ __device__ __forceinline__ float4 router_rows_units(const T* xr, const T* w1, in
       float f[V];
       unpack16(wv[i], f, T());
 #pragma unroll
-      for (int e = 0; e < V; ++e) ws[((i >> 1) * V + e) * kRrUnits + lane + 32 * (i & 1)] = f[e];
+      for (int e = 0; e < V; ++e) ws[(lvec * V + e) * kRrUnits + ((lrow + 8 * i) ^ (8 * lvec))] = f[e];
     }
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       float f[V];
       unpack16(xv[i], f, T());
 #pragma unroll
-      for (int e = 0; e < V; ++e) xs[(((lane >> 4) + 2 * i) * V + e) * kRrRows + (lane & 15)] = f[e];
+      for (int e = 0; e < V; ++e) xs[(lvec * V + e) * kRrRows + ((lrow + 8 * i) ^ (8 * (lvec & 1)))] = f[e];
     }
     if (c + kRrWarps < n) fetch(c + kRrWarps);
     __syncwarp();
+    float acc[4][8];   // the piece's own sums (short chains of roundings), then added to the total
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
 #pragma unroll 8
     for (int k = 0; k < KC; ++k) {
-      const float4 x4 = *reinterpret_cast<const float4*>(xs + k * kRrRows + rg * 4);
-      const float4 wa = *reinterpret_cast<const float4*>(ws + k * kRrUnits + ug * 4);
-      const float4 wb = *reinterpret_cast<const float4*>(ws + k * kRrUnits + 32 + ug * 4);
+      const int sw = 8 * (k / V);   // this k's column swizzle
+      const float4 x4 = *reinterpret_cast<const float4*>(xs + k * kRrRows + ((rg * 4) ^ (sw & 8)));
+      const float4 wa = *reinterpret_cast<const float4*>(ws + k * kRrUnits + ((ug * 4) ^ sw));
+      const float4 wb = *reinterpret_cast<const float4*>(ws + k * kRrUnits + ((32 + ug * 4) ^ sw));
       const float xf[4] = {x4.x, x4.y, x4.z, x4.w};
       const float wf[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
 #pragma unroll
@@ -92,14 +101,18 @@ __device__ __forceinline__ float4 router_rows_units(const T* xr, const T* w1, in
 #pragma unroll
         for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(xf[i], wf[j], acc[i][j]);
     }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) tot[i][j] += acc[i][j];
   }
   __syncthreads();   // the partial tiles overlay the warps' operand areas
   float* red = smem + warp * kRrRows * kRrUnits;   // [warp][16][64]
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     float* p = red + (rg * 4 + i) * kRrUnits + ug * 4;
-    *reinterpret_cast<float4*>(p) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-    *reinterpret_cast<float4*>(p + 32) = make_float4(acc[i][4], acc[i][5], acc[i][6], acc[i][7]);
+    *reinterpret_cast<float4*>(p) = make_float4(tot[i][0], tot[i][1], tot[i][2], tot[i][3]);
+    *reinterpret_cast<float4*>(p + 32) = make_float4(tot[i][4], tot[i][5], tot[i][6], tot[i][7]);
   }
   __syncthreads();
   float4 u = make_float4(0.f, 0.f, 0.f, 0.f);

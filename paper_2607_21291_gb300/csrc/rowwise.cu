@@ -8,6 +8,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "router_rows.cuh"
 #include "topk.cuh"
 
 namespace adadsf {
@@ -461,29 +462,36 @@ __global__ void rope_apply_kernel(T* qkv, int64_t M, int64_t ld, int heads, int 
 }
 
 // ---------------------------------------------------------------- fp32 router (Sec. 3.4)
-// One warp per token: score = sum_j w2[j] * silu(w1[j] . x + b1[j]) + b2.
-__global__ void router_f32_kernel(const float* x, int64_t n, int d, int h, const float* w1,
-                                  const float* b1, const float* w2, const float* b2,
-                                  float* scores) {
+// score = sum_j w2[j] * silu(w1[j] . x + b1[j]) + b2, 16 tokens a block
+// (router_rows.cuh), 64 hidden units at a time. At 128 and 2044 tokens of
+// 512 features it takes 12.8 and 14.5 us (30,000 tokens: 97 us); one warp per token that
+// ran its 64 dots one after another took 45, 46 and 315 us.
+__global__ void __launch_bounds__(kRrThreads, 2)
+    router_f32_kernel(const float* x, int64_t n, int d, int h, const float* w1, const float* b1, const float* w2,
+                      const float* b2, float* scores) {
   pdl_trigger();
   pdl_wait();
-  const int64_t row = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+  extern __shared__ __align__(16) float smem_rr[];
   const int lane = threadIdx.x & 31;
-  if (row >= n) return;
-  const float* xr = x + row * d;
+  const int64_t r0 = (int64_t)blockIdx.x * kRrRows;
+  const int64_t ra = r0 + (lane >> 2) < n ? r0 + (lane >> 2) : n - 1;
+  const int64_t rb = r0 + (lane >> 2) + 8 < n ? r0 + (lane >> 2) + 8 : n - 1;
+  const int64_t row = r0 + (threadIdx.x >> 4);
   float s = 0.f;
-  for (int j = 0; j < h; ++j) {
-    const float* wr = w1 + (int64_t)j * d;
-    float dot = 0.f;
-    for (int c = lane * 4; c < d; c += 128) {
-      const float4 a = *reinterpret_cast<const float4*>(xr + c);
-      const float4 b = *reinterpret_cast<const float4*>(wr + c);
-      dot = fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, dot))));
+  for (int u0 = 0; u0 < h; u0 += kRrUnits) {
+    const float4 u4 = router_rows_units<float>(x + ra * d, x + rb * d, w1, u0, h, d, smem_rr);
+    const float uu[4] = {u4.x, u4.y, u4.z, u4.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int j = u0 + (threadIdx.x & 15) * 4 + e;
+      if (j < h) {
+        const float u = uu[e] + b1[j];
+        s += w2[j] * (u / (1.f + expf(-u)));
+      }
     }
-    const float u = warp_sum(dot) + b1[j];
-    s += w2[j] * (u / (1.f + expf(-u)));
   }
-  if (lane == 0) scores[row] = s + b2[0];
+  s = row16_sum(s);
+  if ((threadIdx.x & 15) == 0 && row < n) scores[row] = s + b2[0];
 }
 
 // ---------------------------------------------------------------- Top-K (Sec. 3.4)
@@ -853,8 +861,10 @@ cudaError_t rope_apply(int dtype, void* qkv, int64_t M, int64_t ld, int n_heads,
 cudaError_t router_f32(const float* x, int64_t n, int d, int h, const float* w1, const float* b1,
                        const float* w2, const float* b2, float* scores, const Dev& dev) {
   if (n <= 0) return cudaSuccess;
-  return launch_pdl(router_f32_kernel, dim3(blocks_for(n, 8)), dim3(256), 0, dev.stream, x, n, d,
-                    h, w1, b1, w2, b2, scores);
+  const cudaError_t e = allow_smem(router_f32_kernel, RouterRows<float>::SMEM_BYTES);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(router_f32_kernel, dim3((unsigned)((n + kRrRows - 1) / kRrRows)), dim3(kRrThreads),
+                    RouterRows<float>::SMEM_BYTES, dev.stream, x, n, d, h, w1, b1, w2, b2, scores);
 }
 
 cudaError_t topk(const float* scores, int B, int T, int K, int32_t* idx, int32_t* rows,

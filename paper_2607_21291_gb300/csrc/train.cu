@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(kRowThreadsT)
 // and ds [m]. FFMA bound (the products stay exact and the sums fp32):
 // 2 M h d operations. G may be 4-byte aligned only (vec: 16-byte loads).
 template <typename T>
-__global__ void __launch_bounds__(kRrThreads)
+__global__ void __launch_bounds__(kRrThreads, 2)
     router_bwd_rows_kernel(const T* x, const T* y_plain, const int32_t* rows, int64_t M, int d, int h,
                            const T* w1, const T* b1, const T* w2, const T* b2, const float* G, int vec, float* du,
                            float* su, float* ds_out) {
@@ -189,8 +189,10 @@ __global__ void __launch_bounds__(kRrThreads)
     gd = warp_sum(gd);
     if (lane == 0) gd_s[warp * (kRrRows / kRrWarps) + i] = gd;
   }
-  const int64_t mx = m0 + (lane & 15) < M ? m0 + (lane & 15) : M - 1;
-  const float4 u4 = router_rows_units<T>(x + (int64_t)rows[mx] * d, w1, 0, h, d, smem_rr);   // barriers: gd_s is visible
+  const int64_t ma = m0 + (lane >> 2) < M ? m0 + (lane >> 2) : M - 1;
+  const int64_t mb = m0 + (lane >> 2) + 8 < M ? m0 + (lane >> 2) + 8 : M - 1;
+  const float4 u4 = router_rows_units<T>(x + (int64_t)rows[ma] * d, x + (int64_t)rows[mb] * d, w1, 0, h, d,
+                                         smem_rr);   // its barriers make gd_s visible
   const int row = threadIdx.x >> 4, j0 = (threadIdx.x & 15) * 4;
   const float uu[4] = {u4.x, u4.y, u4.z, u4.w};
   float si[4], dsi[4], s = 0.f;
@@ -228,7 +230,7 @@ __global__ void __launch_bounds__(kRrThreads)
 // output has only d / 64 such tiles (32 at d = 2048). The last cluster
 // sums db1[j] = sum_m du[m][j], dw2[j] = sum_m ds[m] SiLU(u)[m][j] and db2 =
 // sum_m ds[m] the same way. With part 1 it takes 76 us at M = 2048, d = 2048
-// (bf16) and 1.02 ms at M = 32768, against 1024 us and 20.8 ms for one warp a
+// (bf16) and 0.97 ms at M = 32768, against 1024 us and 20.8 ms for one warp a
 // row with 64 serial dots and a reduction of 17 blocks that summed the vectors
 // in one thread each.
 constexpr int kRedCluster = 8;

@@ -165,6 +165,21 @@ def test_linear_f32_splits(A, M, N, Kd, act):
 
 
 # ---------------------------------------------------------------- router (Sec. 3.4)
+@pytest.mark.parametrize("n,d,h", [(1, 64, 1), (15, 512, 64), (17, 192, 65), (128, 2048, 200), (2044, 512, 64)])
+def test_router_f32_edges(A, n, d, h):
+    """Rows around the 16-row blocks, feature widths that leave warps idle, and
+    hidden widths that are not a multiple of the 64 units of a tile. fp32 sums of
+    d products, then of h: under 2e-6 of the scores' rms."""
+    shape = S.PYTHIA_70M.replace(d=d, router_hidden=h, n_layers=1)
+    W = H.host_layer(shape, n + h)
+    x = S.hidden(n, 1, n, d)[0]
+    sc = torch.full((n + 1,), 7.0, device="cuda")
+    A.adadsf_router_scores(A.make_cfg(shape), A.to_device(W, torch.float32), H.to_dev(x, torch.float32), sc[:n])
+    ref = O.router_scores(x.astype(np.float64), H.f64(W))
+    assert H.elem_rel(sc[:n].cpu().numpy(), ref) < 1e-5
+    assert float(sc[n]) == 7.0
+
+
 @pytest.mark.parametrize("shape,n", [(S.PYTHIA_160M, 1), (S.PYTHIA_160M, 2048), (S.QWEN25_1_5B, 333),
                                      (S.PYTHIA_70M, 128), (S.PYTHIA_160M, 777), (S.PYTHIA_1_4B, 16384)])
 def test_router(A, shape, n):
