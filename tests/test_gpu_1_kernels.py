@@ -281,6 +281,29 @@ def test_attention(A, hq, hkv, hd, B, K, dtype):
         assert H.max_rel(got[b * K:(b + 1) * K], ref) < (2e-2 if dtype == "bf16" else 1e-5)
 
 
+@pytest.mark.parametrize("hq,hkv,hd,B,K", [(8, 8, 64, 1, 65), (8, 2, 64, 3, 128), (2, 1, 128, 2, 383), (1, 1, 64, 1, 700)])
+def test_attention_f32_tiles(A, hq, hkv, hd, B, K):
+    """Key and query tiles of 64 of the fp32 kernel, and causality to the bit: an
+    infinite value and a NaN key of the last token leave every earlier row as it
+    was. fp32 softmax and sums over K keys: within 1e-5 of the largest element."""
+    shape = S.PYTHIA_160M.replace(n_heads=hq, n_kv_heads=hkv, head_dim=hd, d=hq * hd, dtype="f32")
+    width = (hq + 2 * hkv) * hd
+    g = np.random.default_rng(B * K + hq)
+    qkv = g.standard_normal((B * K, width)).astype(np.float32)
+    out = torch.empty((B * K, hq * hd), device="cuda")
+    A.adadsf_causal_attention(A.make_cfg(shape), H.to_dev(qkv, torch.float32), B, K, out)
+    for b in range(B):
+        blk = qkv[b * K:(b + 1) * K].astype(np.float64)
+        ref = O.causal_attention(blk[:, :hq * hd], blk[:, hq * hd:(hq + hkv) * hd], blk[:, (hq + hkv) * hd:],
+                                 hq, hkv, hd)
+        assert H.max_rel(out[b * K:(b + 1) * K].cpu().numpy(), ref) < 1e-5
+    qkv.reshape(B, K, width)[:, -1, (hq + hkv) * hd:] = np.inf
+    qkv.reshape(B, K, width)[:, -1, hq * hd:(hq + hkv) * hd] = np.nan
+    again = torch.empty_like(out)
+    A.adadsf_causal_attention(A.make_cfg(shape), H.to_dev(qkv, torch.float32), B, K, again)
+    assert torch.equal(again.view(B, K, -1)[:, :-1], out.view(B, K, -1)[:, :-1])
+
+
 @pytest.mark.parametrize("hq,hkv,hd,B,K", [(12, 12, 64, 7, 520), (12, 12, 64, 7, 300), (12, 2, 128, 5, 520),
                                           (4, 4, 128, 20, 300), (28, 4, 128, 2, 1100)])
 def test_attention_paired_tiles(A, hq, hkv, hd, B, K):
