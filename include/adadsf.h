@@ -244,8 +244,9 @@ adadsf_status adadsf_fold_norms(const adadsf_model_cfg *cfg, const adadsf_layer_
  * softmax over n_classes of the logits h W_head^T (w_head_dev [n_classes, d],
  * e.g. the tied embedding); acc_dev[0] += sum of the rows' KL, acc_dev[1] +=
  * n_rows. Logits are fp32 (workspace: adadsf_align_workspace_size(n_rows,
- * n_classes), 8 n_rows n_classes bytes of them: call on row chunks for large
- * vocabularies). bf16 needs d and n_classes multiples of 64.
+ * n_classes), 8 n_rows n_classes bytes with room for all of them, which the
+ * fp32 path stores; bf16 keeps sums per row there instead: call on row chunks
+ * for large vocabularies). bf16 needs d and n_classes multiples of 64.
  * Eq. 11 is L_align + (1/L) sum_l L_hid^(l) of those accumulators.
  * Sums run in a fixed order (bit-reproducible).
  * ---------------------------------------------------------------------- */

@@ -1144,19 +1144,21 @@ adadsf_status adadsf_align_output(const void* hs_dev, const void* hd_dev, const 
   const size_t part = cv.take((size_t)train_row_blocks(n_rows) * 8);
   const size_t ls = cv.take((size_t)n_rows * n_classes * 4);
   const size_t ld = cv.take((size_t)n_rows * n_classes * 4);
-  // logits h W_head^T of both models, fp32
+  if (dtype == ADADSF_BF16)
+    // both products and the loss in one kernel; its records (at most 10 floats
+    // per row and started 128 classes) lie where the fp32 path keeps logits
+    return launch(dev, ADADSF_KERNEL_ALIGN, true, 4.0 * n_rows * n_classes * d,
+                  (2.0 * n_rows * d + (double)n_classes * d) * 2.0,
+                  CALL(kl_tc(hs_dev, hd_dev, w_head_dev, n_rows, d, n_classes, at<float>(ws, ls), at<double>(ws, part),
+                             acc_dev, dev),
+                       "output alignment"));
+  // fp32: logits h W_head^T of both models, then the loss over them
   for (int k = 0; k < 2; ++k) {
     GemmArgs g = linear_args(k == 0 ? hs_dev : hd_dev, d, w_head_dev, n_rows, n_classes, d);
-    float* lg = at<float>(ws, k == 0 ? ls : ld);
-    if (dtype == ADADSF_BF16) {
-      g.epi.out_f32 = lg;
-      g.epi.ld_out = n_classes;
-    } else {
-      g.epi.out = lg;
-      g.epi.ld_out = n_classes;
-    }
-    TRY(launch(dev, ADADSF_KERNEL_LINEAR, dtype == ADADSF_BF16, 2.0 * n_rows * n_classes * d,
-               ((double)n_rows * d + (double)n_classes * d) * elem_size(dtype) + 4.0 * n_rows * n_classes,
+    g.epi.out = at<float>(ws, k == 0 ? ls : ld);
+    g.epi.ld_out = n_classes;
+    TRY(launch(dev, ADADSF_KERNEL_LINEAR, false, 2.0 * n_rows * n_classes * d,
+               ((double)n_rows * d + (double)n_classes * d + (double)n_rows * n_classes) * 4.0,
                [&] { return run_linear(dtype, g, dev, "head logits"); }));
   }
   return launch(dev, ADADSF_KERNEL_ALIGN, false, 0, 8.0 * n_rows * n_classes,

@@ -75,9 +75,6 @@ struct Epilogue {
   int cos_ld = 0;
   const void* cos_in = nullptr;
   int64_t ld_cos_in = 0;
-  // fp32 output instead of `out` (bf16 path, no residual): out_f32[row][n],
-  // leading dimension ld_out (the logits of the output alignment, Eq. 10)
-  float* out_f32 = nullptr;
 };
 
 // acc = A . W^T (+ A2 . Wk2^T when K2 > 0: a second K source, bf16
@@ -136,6 +133,13 @@ cudaError_t kl_rows(const float* ls, const float* ld, int64_t n_rows, int n_cls,
 cudaError_t router_backward(int dtype, const void* x, const void* y_plain, const int32_t* rows, int64_t M, int d,
                             int h, const void* w1, const void* b1, const void* w2, const void* b2, const float* G,
                             float* du, float* su, float* ds, float* grad, const Dev& dev);
+// acc[0] += sum of nblocks doubles in a fixed order, acc[1] += count.
+cudaError_t sum_partials(const double* partials, int nblocks, int64_t count, double* acc, const Dev& dev);
+// kl_tc.cu -- Eq. 10 from bf16 hidden states and head on tcgen05, logits never
+// stored. rec: fp32 scratch, 10 floats per row and started 128 classes; partials:
+// train_row_blocks(n_rows) doubles.
+cudaError_t kl_tc(const void* hs, const void* hd, const void* w, int64_t n_rows, int d, int n_cls, float* rec,
+                  double* partials, double* acc, const Dev& dev);
 // gemm_simt.cu -- fp32 projections on CUDA cores.
 cudaError_t gemm_f32(const GemmArgs& a, const Dev& dev);
 

@@ -108,7 +108,8 @@ __global__ void __launch_bounds__(kRowThreadsT)
 }
 
 // Eq. 10 per row (one warp): KL(softmax(ld) || softmax(ls)) over n_cls
-// classes, from fp32 logits.
+// classes, from fp32 logits (fp32 storage; bf16 folds the logits into the
+// sums where they are computed, kl_tc.cu).
 __global__ void __launch_bounds__(kRowThreadsT)
     kl_rows_kernel(const float* ls, const float* ld, int64_t n_rows, int n_cls, double* partials) {
   pdl_trigger();
@@ -383,6 +384,10 @@ cudaError_t router_backward_t(const void* x, const void* y_plain, const int32_t*
 
 int train_row_blocks(int64_t n) { return row_blocks(n); }
 
+cudaError_t sum_partials(const double* partials, int nblocks, int64_t count, double* acc, const Dev& dev) {
+  return launch_pdl(sum_partials_kernel, dim3(1), dim3(256), 0, dev.stream, partials, nblocks, count, acc);
+}
+
 cudaError_t align_hidden(int dtype, const void* hs, const void* hd, int64_t n_rows, int d, float* grad,
                          double* partials, double* acc, const Dev& dev) {
   if (n_rows <= 0) return cudaSuccess;
@@ -395,8 +400,7 @@ cudaError_t align_hidden(int dtype, const void* hs, const void* hd, int64_t n_ro
     e = launch_pdl(align_hidden_kernel<float>, dim3(nb), dim3(kRowThreadsT), 0, dev.stream,
                    static_cast<const float*>(hs), static_cast<const float*>(hd), n_rows, d, grad, partials);
   if (e != cudaSuccess) return e;
-  return launch_pdl(sum_partials_kernel, dim3(1), dim3(256), 0, dev.stream, (const double*)partials, nb, n_rows,
-                    acc);
+  return sum_partials(partials, nb, n_rows, acc, dev);
 }
 
 cudaError_t kl_rows(const float* ls, const float* ld, int64_t n_rows, int n_cls, double* partials, double* acc,
@@ -406,8 +410,7 @@ cudaError_t kl_rows(const float* ls, const float* ld, int64_t n_rows, int n_cls,
   cudaError_t e = launch_pdl(kl_rows_kernel, dim3(nb), dim3(kRowThreadsT), 0, dev.stream, ls, ld, n_rows, n_cls,
                              partials);
   if (e != cudaSuccess) return e;
-  return launch_pdl(sum_partials_kernel, dim3(1), dim3(256), 0, dev.stream, (const double*)partials, nb, n_rows,
-                    acc);
+  return sum_partials(partials, nb, n_rows, acc, dev);
 }
 
 cudaError_t router_backward(int dtype, const void* x, const void* y_plain, const int32_t* rows, int64_t M, int d,

@@ -59,6 +59,31 @@ def test_align_output(A, n, d, V, dtype):
     assert abs(same.cpu().numpy()[0]) < 1e-5 * n                # KL(P || P) = 0
 
 
+@pytest.mark.parametrize("n,d,V,scale", [(1, 64, 64, 1.0), (127, 64, 192, 4.0), (129, 128, 19456, 1.0),
+                                          (300, 320, 25664, 3.0), (1300, 64, 64, 1.0)])
+def test_align_output_tiles(A, n, d, V, scale):
+    """bf16: rows and classes around the 128 x 128 tiles, row blocks that start
+    inside a CTA's range of tiles, a last tile of 64 classes, and logits wide
+    enough that the running maxima move. The logits are fp32 sums of exact
+    products (a few 1e-6 relative), so the loss holds to 1e-4 of its value; twice
+    the same bits."""
+    g = np.random.default_rng(n + V)
+    hs = S.round_to(g.standard_normal((n, d)).astype(np.float32), "bf16")
+    hd = S.round_to((hs + 0.3 * g.standard_normal((n, d))).astype(np.float32), "bf16")
+    W = S.round_to((g.standard_normal((V, d)) * scale / np.sqrt(d)).astype(np.float32), "bf16")
+    args = [H.to_dev(a, torch.bfloat16) for a in (hs, hd, W)]
+    ws = A.workspace(A.lib().adadsf_align_workspace_size(n, V))
+    vals = []
+    for _ in range(2):
+        acc = torch.zeros(2, dtype=torch.float64, device="cuda")
+        A.adadsf_align_output(*args, acc, ws=ws)
+        assert A.adadsf_sync_check(ws) == A.OK
+        vals.append(acc.cpu().numpy().tolist())
+    ref = O.output_alignment(hs.astype(np.float64), hd.astype(np.float64), W.astype(np.float64))
+    assert vals[0][1] == n and vals[0] == vals[1]
+    assert vals[0][0] == pytest.approx(ref.sum(), rel=1e-4)
+
+
 QWEN_SMALL = S.QWEN25_1_5B.replace(d=1024, n_heads=8, n_kv_heads=2, ffn=1536, n_layers=1)
 
 
