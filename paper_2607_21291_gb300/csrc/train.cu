@@ -41,21 +41,23 @@ __global__ void sum_partials_kernel(const double* partials, int nblocks, int64_t
 }
 
 // Per-block fixed-order sum of the warps' per-row values.
+template <int THREADS = kRowThreadsT>
 __device__ __forceinline__ void block_partial(double mine, double* partials) {
-  __shared__ double red[kRowThreadsT / 32];
+  __shared__ double red[THREADS / 32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (lane == 0) red[w] = mine;
   __syncthreads();
   if (threadIdx.x == 0) {
     double s = 0;
-    for (int i = 0; i < kRowThreadsT / 32; ++i) s += red[i];
+    for (int i = 0; i < THREADS / 32; ++i) s += red[i];
     partials[blockIdx.x] = s;
   }
 }
 
 // Eq. 9 per row (one warp): n = |softmax(hs) - softmax(hd)| over the d
 // features, and, with grad, d n / d hs = p (r / n - p . r / n) (0 if n = 0),
-// p = softmax(hs), r = p - softmax(hd). fp32, four passes over the rows.
+// p = softmax(hs), r = p - softmax(hd). fp32, four passes over the rows: the
+// general path, for any d and alignment (align_hidden_vec_kernel otherwise).
 template <typename T>
 __global__ void __launch_bounds__(kRowThreadsT)
     align_hidden_kernel(const T* hs, const T* hd, int64_t n_rows, int d, float* grad, double* partials) {
@@ -105,6 +107,117 @@ __global__ void __launch_bounds__(kRowThreadsT)
     }
   }
   block_partial(mine, partials);
+}
+
+// The same with rows held in registers: 128 threads a row (one warp for rows of
+// at most two 16-byte vectors a lane), NV vectors of each input a thread, loaded
+// once, and each element's two exponentials computed once instead of three
+// times. Three exchanges a row (maxima, sums, norm and projection). What bounds it
+// is HBM: 2 n d values read and, with grad, n d floats written. At 4096 rows of
+// 2048 (bf16) it takes 25 us with the gradient and 21 us without, the sum over blocks
+// included (47 and 27 us on the general path: element-wise loads, one warp a row).
+// Needs d a multiple of a vector's elements and 16-byte aligned pointers.
+constexpr int kAlignThreads = 512;
+
+template <typename T, int G, int NV>
+__global__ void __launch_bounds__(kAlignThreads)
+    align_hidden_vec_kernel(const T* hs, const T* hd, int64_t n_rows, int d, float* grad, double* partials) {
+  pdl_trigger();
+  pdl_wait();
+  constexpr int V = Elem<T>::kVec, GROUPS = kAlignThreads / G, W = G / 32;
+  __shared__ float2 xch[3][GROUPS][W];
+  const int grp = threadIdx.x / G, gt = threadIdx.x % G;
+  const int gw = gt >> 5, lane = threadIdx.x & 31;
+  // a pair of values over the group's warps; each of the three slots is reused only
+  // after the barriers of the other two
+  auto exchange = [&](int slot, float2 v, auto op) {
+    if (W == 1) return v;
+    if (lane == 0) xch[slot][grp][gw] = v;
+    named_bar_sync(1 + grp, G);
+    v = xch[slot][grp][0];
+#pragma unroll
+    for (int w = 1; w < W; ++w) {
+      const float2 f = xch[slot][grp][w];
+      v = make_float2(op(v.x, f.x), op(v.y, f.y));
+    }
+    return v;
+  };
+  const auto fmx = [](float a, float b) { return fmaxf(a, b); };
+  const auto fad = [](float a, float b) { return a + b; };
+  const int64_t step = (int64_t)gridDim.x * GROUPS;
+  double mine = 0;
+  for (int64_t r = (int64_t)blockIdx.x * GROUPS + grp; r < n_rows; r += step) {
+    const T* a = hs + r * d;
+    const T* b = hd + r * d;
+    float ea[NV][V], eb[NV][V];
+    float ma = -INFINITY, mb = -INFINITY;
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const int k = (i * G + gt) * V;
+      if (k < d) {
+        load_vec(a + k, ea[i]);
+        load_vec(b + k, eb[i]);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < NV; ++i)
+      if ((i * G + gt) * V < d)
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+          ma = fmaxf(ma, ea[i][e]);
+          mb = fmaxf(mb, eb[i][e]);
+        }
+    for (int o = 16; o > 0; o >>= 1) {
+      ma = fmaxf(ma, __shfl_xor_sync(0xffffffffu, ma, o));
+      mb = fmaxf(mb, __shfl_xor_sync(0xffffffffu, mb, o));
+    }
+    const float2 m2 = exchange(0, make_float2(ma, mb), fmx);
+    float za = 0.f, zb = 0.f;
+#pragma unroll
+    for (int i = 0; i < NV; ++i)
+      if ((i * G + gt) * V < d)
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+          ea[i][e] = expf(ea[i][e] - m2.x);
+          eb[i][e] = expf(eb[i][e] - m2.y);
+          za += ea[i][e];
+          zb += eb[i][e];
+        }
+    const float2 z2 = exchange(1, make_float2(warp_sum(za), warp_sum(zb)), fad);
+    const float ia = 1.f / z2.x, ib = 1.f / z2.y;
+    float n2 = 0.f, pr = 0.f;
+#pragma unroll
+    for (int i = 0; i < NV; ++i)
+      if ((i * G + gt) * V < d)
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+          const float p = ea[i][e] * ia;
+          const float rr = p - eb[i][e] * ib;
+          n2 = fmaf(rr, rr, n2);
+          pr = fmaf(p, rr, pr);
+          ea[i][e] = p;
+          eb[i][e] = rr;
+        }
+    const float2 s2 = exchange(2, make_float2(warp_sum(n2), warp_sum(pr)), fad);
+    const float n = sqrtf(s2.x);
+    if (gt == 0) mine += (double)n;
+    if (grad) {
+      const float in = n > 0.f ? 1.f / n : 0.f;
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        const int k = (i * G + gt) * V;
+        if (k < d) {
+          float* g = grad + r * d + k;
+#pragma unroll
+          for (int e = 0; e < V; e += 4)
+            *reinterpret_cast<float4*>(g + e) =
+                make_float4(ea[i][e] * (eb[i][e] - s2.y) * in, ea[i][e + 1] * (eb[i][e + 1] - s2.y) * in,
+                            ea[i][e + 2] * (eb[i][e + 2] - s2.y) * in, ea[i][e + 3] * (eb[i][e + 3] - s2.y) * in);
+        }
+      }
+    }
+  }
+  block_partial<kAlignThreads>(mine, partials);
 }
 
 // Eq. 10 per row (one warp): KL(softmax(ld) || softmax(ls)) over n_cls
@@ -380,6 +493,31 @@ cudaError_t router_backward_t(const void* x, const void* y_plain, const int32_t*
                             (const float*)ds, grad);
 }
 
+// Rows in registers where a row is whole 16-byte vectors of aligned memory, fits
+// (one warp up to 2 vectors a lane, else 128 threads up to 4) and gives at least
+// half of a warp's lanes a vector; the general kernel otherwise (100,000 rows
+// of 64 without gradient: 41.8 us there, 43.6 us with 8 lanes of 32 at work).
+template <typename T>
+cudaError_t align_hidden_t(const T* hs, const T* hd, int64_t n_rows, int d, float* grad, double* partials, int nb,
+                           const Dev& dev) {
+  constexpr int V = Elem<T>::kVec;
+  const bool vec = d % V == 0 && d / V >= 16 && ((reinterpret_cast<uintptr_t>(hs) | reinterpret_cast<uintptr_t>(hd) |
+                                   reinterpret_cast<uintptr_t>(grad)) & 15u) == 0;
+  const int nv32 = (d / V + 31) / 32, nv128 = (d / V + 127) / 128;
+  const dim3 g((unsigned)nb), b(kAlignThreads);
+  if (vec && nv32 == 1)
+    return launch_pdl(align_hidden_vec_kernel<T, 32, 1>, g, b, 0, dev.stream, hs, hd, n_rows, d, grad, partials);
+  if (vec && nv32 == 2)
+    return launch_pdl(align_hidden_vec_kernel<T, 32, 2>, g, b, 0, dev.stream, hs, hd, n_rows, d, grad, partials);
+  if (vec && nv128 == 1)
+    return launch_pdl(align_hidden_vec_kernel<T, 128, 1>, g, b, 0, dev.stream, hs, hd, n_rows, d, grad, partials);
+  if (vec && nv128 == 2)
+    return launch_pdl(align_hidden_vec_kernel<T, 128, 2>, g, b, 0, dev.stream, hs, hd, n_rows, d, grad, partials);
+  if (vec && nv128 <= 4)
+    return launch_pdl(align_hidden_vec_kernel<T, 128, 4>, g, b, 0, dev.stream, hs, hd, n_rows, d, grad, partials);
+  return launch_pdl(align_hidden_kernel<T>, g, dim3(kRowThreadsT), 0, dev.stream, hs, hd, n_rows, d, grad, partials);
+}
+
 }  // namespace
 
 int train_row_blocks(int64_t n) { return row_blocks(n); }
@@ -392,13 +530,11 @@ cudaError_t align_hidden(int dtype, const void* hs, const void* hd, int64_t n_ro
                          double* partials, double* acc, const Dev& dev) {
   if (n_rows <= 0) return cudaSuccess;
   const int nb = row_blocks(n_rows);
-  cudaError_t e;
-  if (dtype == kBF16)
-    e = launch_pdl(align_hidden_kernel<bf16>, dim3(nb), dim3(kRowThreadsT), 0, dev.stream,
-                   static_cast<const bf16*>(hs), static_cast<const bf16*>(hd), n_rows, d, grad, partials);
-  else
-    e = launch_pdl(align_hidden_kernel<float>, dim3(nb), dim3(kRowThreadsT), 0, dev.stream,
-                   static_cast<const float*>(hs), static_cast<const float*>(hd), n_rows, d, grad, partials);
+  const cudaError_t e = dtype == kBF16
+                            ? align_hidden_t(static_cast<const bf16*>(hs), static_cast<const bf16*>(hd), n_rows, d, grad,
+                                             partials, nb, dev)
+                            : align_hidden_t(static_cast<const float*>(hs), static_cast<const float*>(hd), n_rows, d,
+                                             grad, partials, nb, dev);
   if (e != cudaSuccess) return e;
   return sum_partials(partials, nb, n_rows, acc, dev);
 }

@@ -40,6 +40,36 @@ def test_align_hidden(A, n, d, dtype):
     assert again.cpu().numpy().tolist() == got.tolist()        # fixed summation order
 
 
+@pytest.mark.parametrize("n,d,dtype,shift", [(9, 256, "bf16", 0), (33, 512, "bf16", 0), (17, 520, "bf16", 0),
+                                              (70, 2056, "bf16", 0), (5, 4096, "bf16", 0), (5, 4104, "bf16", 0),
+                                              (12, 2048, "f32", 0), (12, 250, "f32", 0), (31, 1000, "f32", 1),
+                                              (20000, 64, "bf16", 0)])
+def test_align_hidden_widths(A, n, d, dtype, shift):
+    """Row widths on both sides of every register layout (one warp or 128
+    threads a row, one to four vectors a thread) and of the general path (width
+    not whole vectors, too wide, gradient at an odd float). Softmax sums of d
+    fp32 terms: 2e-5 of the largest gradient element. An element p (r - p.r) / n
+    carries a few 2^-24 of p whatever r - p.r leaves of it, and the largest p are
+    up to a few thousand times the gradient's rms: under 1e-3 of the rms.
+    Twice the same bits."""
+    g = np.random.default_rng(n + d)
+    hs = S.round_to(g.standard_normal((n, d)).astype(np.float32) * 2, dtype)
+    hd = S.round_to((hs + 0.5 * g.standard_normal((n, d))).astype(np.float32), dtype)
+    td = torch.bfloat16 if dtype == "bf16" else torch.float32
+    acc = torch.zeros(2, dtype=torch.float64, device="cuda")
+    store = torch.full((n * d + 8,), 7.0, device="cuda")
+    grad = store[shift:shift + n * d].view(n, d)
+    A.adadsf_align_hidden(H.to_dev(hs, td), H.to_dev(hd, td), acc, grad)
+    ref = O.hidden_alignment(hs.astype(np.float64), hd.astype(np.float64))
+    assert acc.cpu().numpy()[0] == pytest.approx(ref.sum(), rel=1e-5) and float(acc[1]) == n
+    H.assert_close(grad.cpu().numpy(), O.hidden_alignment_grad(hs.astype(np.float64), hd.astype(np.float64)), 2e-5,
+                   "grad", elem_tol=1e-3)
+    assert float(store[shift + n * d]) == 7.0                   # nothing past the last row
+    again = torch.zeros(2, dtype=torch.float64, device="cuda")
+    A.adadsf_align_hidden(H.to_dev(hs, td), H.to_dev(hd, td), again, grad)
+    assert again.cpu().numpy().tolist() == acc.cpu().numpy().tolist()
+
+
 @pytest.mark.parametrize("n,d,V,dtype", [(64, 1024, 2048, "bf16"), (5, 64, 128, "bf16"), (33, 512, 1000, "f32"),
                                          (300, 768, 6272, "bf16")])
 def test_align_output(A, n, d, V, dtype):
