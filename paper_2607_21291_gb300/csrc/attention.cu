@@ -59,7 +59,6 @@ __global__ void __launch_bounds__(kAtThreads) attn_f32_kernel(const float* qkv, 
                                                               int K, int n_heads, int n_kv, int B, float scale) {
   using C = AttnF32<HD>;
   constexpr int NO = HD / 64;   // 16-byte pieces of a thread's output columns
-  pdl_trigger();
   extern __shared__ __align__(16) float smem_at[];
   float* sQ = smem_at;
   float* sK = sQ + kAtQ * C::LD;
@@ -86,6 +85,7 @@ __global__ void __launch_bounds__(kAtThreads) attn_f32_kernel(const float* qkv, 
   };
   const int64_t kc0 = (int64_t)n_heads * HD + (int64_t)g * HD, vc0 = kc0 + (int64_t)n_kv * HD;
   pdl_wait();
+  pdl_trigger();
   load_rows(sQ, C::LD, (int64_t)h * HD, q0);
   load_rows(sK, C::LD, kc0, 0);
   load_rows(sV, HD, vc0, 0);

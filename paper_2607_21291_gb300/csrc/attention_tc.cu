@@ -171,7 +171,6 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   const int nqb = (p.K + kQB - 1) / kQB;
   const int n_items = p.Hq * p.B * (p.pair ? (nqb + 1) / 2 : nqb);
 
-  pdl_trigger();
   if (threadIdx.x == 0) {
     mbar_init(q_full, 1);
     mbar_init(q_empty, 1);
@@ -250,6 +249,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           ++issued;
         }
       }
+      if (kprod) pdl_trigger();
       // drain: the copies issued last into each stage (and the last Q) have landed
       if (kprod && it > 0) mbar_wait_drain(q_full, (it - 1) & 1, p.timeout_ns);
       for (int st = 0; st < NST && st < issued; ++st) {
@@ -521,8 +521,8 @@ __global__ void __launch_bounds__(kVtThreads)
     vt_transpose_kernel(const bf16* qkv, int64_t ld, int col0, int B, int K, int Hkv, int hd,
                         int pad, bf16* vt) {
   __shared__ uint32_t tile[kVtTile * kVtLd];   // [j][e], two bf16 per word
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const uint16_t* tile16 = reinterpret_cast<const uint16_t*>(tile);
   const int ntj = (K + kVtTile - 1) / kVtTile, nte = (hd + kVtTile - 1) / kVtTile;
   const int64_t ntiles = (int64_t)ntj * nte * B * Hkv;

@@ -107,6 +107,15 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
 // Every kernel calls pdl_wait() before its first global access that can depend
 // on (or conflict with) earlier kernels. Without the launch attribute both are
 // no-ops.
+// Where the trigger stands: a successor's CTAs that wait beside a running kernel
+// slow it (a 133 us tensor-core kernel took 38 us more with 125 small blocks
+// waiting from its start on), and a waiting kernel that has triggered lets the one
+// after it in as well. So no kernel triggers before its own pdl_wait() has
+// returned, and the tensor-core kernels trigger when their producer has issued its
+// last loads, which still leaves the successor's launch latency under the last
+// products and the epilogue. Against a trigger at every kernel's entry: a layer of the
+// Qwen2.5-1.5B shape on one sequence of 777 tokens 119.7 -> 108.5 us, the Pythia-160M
+// forward 698 -> 640 us, a fp32 Pythia-70M layer 77.8 -> 69.0 us.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -37,8 +37,8 @@ constexpr int kRopeThreads = 1024;       // rotary + cache append: threads per s
 template <typename T>
 __global__ void kv_fill_kernel(const T* qkv, int64_t ld, int q, int kvw, int B, int K, int hd,
                                int C_max, T* kc, T* vc) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   constexpr int V = Elem<T>::kVec;
   const int nvec = kvw / V;                       // 16-byte vectors of one row's keys
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -56,8 +56,8 @@ __global__ void kv_fill_kernel(const T* qkv, int64_t ld, int q, int kvw, int B, 
 // kept positions (+inf when K = 0). One block per sequence.
 __global__ void kv_threshold_kernel(const float* scores, const int32_t* idx, int T, int K,
                                     int32_t* lens, float* thr) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ float red[32];
   __shared__ int any_nan;
   const int b = blockIdx.x;
@@ -80,8 +80,8 @@ __global__ void kv_threshold_kernel(const float* scores, const int32_t* idx, int
 }
 
 __global__ void cache_header_kernel(int32_t* hdr, int T, int C_max, int L, int B) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   if (threadIdx.x == 0) {
     hdr[0] = T;
     hdr[1] = C_max;
@@ -100,8 +100,8 @@ __global__ void cache_header_kernel(int32_t* hdr, int T, int C_max, int L, int B
 // router is not forked onto a stream of its own.)
 __global__ void decode_decide_kernel(const float* scores, const float* thr, const int32_t* hdr, int B,
                                      int C_max, int32_t* rows, int32_t* pos, int32_t* kept_out, int* err) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B) return;
   int t = hdr[0];
@@ -133,8 +133,8 @@ __global__ void __launch_bounds__(kDecThreads)
     decode_attn_f32_kernel(const float* qkv, int64_t ld, int Hq, int Hkv, int hd, const float* kc,
                            const float* vc, const int32_t* lens, int C_max, int nsplit, float scale_log2,
                            float* part_o, float2* part_ml) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int s = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
   const int G = Hq / Hkv;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -282,8 +282,8 @@ __global__ void __launch_bounds__(kDecTcThreads)
     tma_prefetch_desc(&tv);
   }
   __syncthreads();
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   int n = lens[b];
   n = n < 0 ? 0 : (n > C_max ? C_max : n);
   int lo, hi;
@@ -448,8 +448,8 @@ __global__ void __launch_bounds__(kDecTcThreads)
 template <typename T>
 __global__ void decode_combine_kernel(const float* part_o, const float2* part_ml, int Hq, int hd,
                                       int nsplit, T* out, int64_t ld_out) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int hq = blockIdx.x, b = blockIdx.y;
   const int64_t slot0 = ((int64_t)b * Hq + hq) * nsplit;
   float m = -INFINITY;
@@ -476,8 +476,8 @@ template <typename T>
 __global__ void __launch_bounds__(kRopeThreads) rope_append_kernel(T* qkv, int64_t ld, int Hq, int Hkv, int hd, int half,
                                    const int32_t* pos, const float2* tab, const int32_t* rows,
                                    int32_t* lens, int C_max, T* kc, T* vc, int* err) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int b = blockIdx.x;
   T* row = qkv + (int64_t)b * ld;
   const int q = Hq * hd, kvw = Hkv * hd;
@@ -519,8 +519,8 @@ __global__ void __launch_bounds__(kRopeThreads) rope_append_kernel(T* qkv, int64
 }
 
 __global__ void decode_advance_kernel(int32_t* hdr) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   if (threadIdx.x == 0) hdr[0] += 1;
 }
 

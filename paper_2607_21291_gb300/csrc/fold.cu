@@ -14,8 +14,8 @@ namespace {
 // c[n] += W[n, :] . b  (one warp per row of W, fp32 sums, one rounding)
 template <typename T>
 __global__ void fold_bias_kernel(const T* w, int N, int K, const T* b, T* c) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int n = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
   const int lane = threadIdx.x & 31;
   if (n >= N) return;
@@ -28,8 +28,8 @@ __global__ void fold_bias_kernel(const T* w, int N, int K, const T* b, T* c) {
 // W[n, k] *= g[k] in place (one rounding to the storage type)
 template <typename T>
 __global__ void fold_scale_kernel(T* w, int64_t N, int K, const T* g) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N * K) return;
   const int k = (int)(i % K);
@@ -38,8 +38,8 @@ __global__ void fold_scale_kernel(T* w, int64_t N, int K, const T* g) {
 
 template <typename T>
 __global__ void fill_kernel(T* v, int n, float value) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) v[i] = Elem<T>::from_f(value);
 }

@@ -118,7 +118,6 @@ __global__ void __launch_bounds__(F32Tile<BM, BN, TM, TN, KS>::THREADS, 2) gemm_
   constexpr int LOADS = (BM + BN) * 8 / C::THREADS;
   constexpr int LROWS = C::THREADS / 8;            // rows a loading step covers
   extern __shared__ __align__(16) float smem_f32[];
-  pdl_trigger();
   const int tid = threadIdx.x;
   const int num_n = (p.N + NOUT - 1) / NOUT;
   const int tile = (int)(blockIdx.x / S), rank = (int)(blockIdx.x % S);
@@ -153,6 +152,7 @@ __global__ void __launch_bounds__(F32Tile<BM, BN, TM, TN, KS>::THREADS, 2) gemm_
     }
   };
   pdl_wait();
+  pdl_trigger();
 #pragma unroll
   for (int s = 0; s < kF32Stages - 1; ++s) {
     if (kb0 + s < kb1) load_stage(kb0 + s, s);

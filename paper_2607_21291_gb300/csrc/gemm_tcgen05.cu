@@ -701,7 +701,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int tiles0 = tiles_of(p, BM);
   const int num_tiles = tiles0 + tiles_of(p2, BM);
 
-  pdl_trigger();
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::STAGES; ++s) {
       mbar_init(full0 + 8 * s, 1);
@@ -780,6 +779,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         first = false;
         if (!ok) break;
       }
+      pdl_trigger();
       // Drain: wait until the last copy issued into each stage has landed.
       for (int s = 0; s < C::STAGES; ++s) {
         if (issued <= s) break;
@@ -910,7 +910,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int kb1 = (rank + 1) * ti.nkb / S;
   const int nkb = kb1 - kb0;
 
-  pdl_trigger();
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::STAGES; ++s) {
       mbar_init(full0 + 8 * s, 1);
@@ -984,6 +983,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         ++issued;
         if (++stage == C::STAGES) { stage = 0; phase ^= 1; }
       }
+      pdl_trigger();
       for (int s = 0; s < C::STAGES; ++s) {
         if (issued <= s) break;
         const int last = s + ((issued - 1 - s) / C::STAGES) * C::STAGES;
@@ -1120,7 +1120,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     return DUAL ? (rank == 1 ? &tmB2 : &tmB) : s.b;
   };
 
-  pdl_trigger();
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::STAGES; ++s) {
       mbar_init(full0 + 8 * s, 1);              // the even CTA's producer arms both CTAs' bytes
@@ -1203,6 +1202,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       first = false;
       if (!ok) break;
     }
+    pdl_trigger();
     // Drain (even CTA, whose full barriers count both CTAs' copies).
     if (lane == 0 && rank == 0) {
       for (int s = 0; s < C::STAGES; ++s) {
@@ -1259,6 +1259,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         first = false;
         if (!ok) break;
       }
+      pdl_trigger();
       // Drain (even CTA, whose full barriers count both CTAs' copies).
       if (rank == 0) {
         for (int s = 0; s < C::STAGES; ++s) {

@@ -284,8 +284,8 @@ __global__ void __launch_bounds__(kKlThreads, 1)
 // block, in a fixed order. A half without a class (ms = md = -inf, sums 0) adds nothing.
 __global__ void __launch_bounds__(256)
     kl_merge_kernel(const float* rec, int M, int num_n, int64_t tiles, int G, double* partials) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ double red[8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double mine = 0.0;

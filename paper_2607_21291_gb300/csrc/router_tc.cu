@@ -124,7 +124,6 @@ __global__ void __launch_bounds__(kRThreads, 1)
   const int64_t u0 = unit_start(blockIdx.x, p);
   const int64_t u1 = unit_start((int64_t)blockIdx.x + 1, p);
 
-  pdl_trigger();
   if (threadIdx.x == 0) {
     for (int s = 0; s < kRStages; ++s) {
       mbar_init(full0 + 8 * s, 1);
@@ -180,6 +179,7 @@ __global__ void __launch_bounds__(kRThreads, 1)
         ++issued;
         if (++stage == kRStages) { stage = 0; phase ^= 1; }
       }
+      pdl_trigger();
       // Drain: wait until the last copy issued into each stage has landed.
       for (int s = 0; s < kRStages; ++s) {
         if (issued <= s) break;

@@ -20,8 +20,8 @@ constexpr int kMaxChunks = 16;  // per-lane 16-byte vectors held in registers (d
 template <typename T>
 __global__ void embed_kernel(const int32_t* ids, int64_t n, const T* table, int vocab, int d,
                              T* out, int* err) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   constexpr int V = Elem<T>::kVec;
   const int64_t row = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
   const int lane = threadIdx.x & 31;
@@ -187,11 +187,11 @@ template <typename T, bool RMS, int NCH>
 __global__ void __launch_bounds__(32 * kFewRowWarps)
     norm_few_rows_kernel(const T* x, const int32_t* rows, int64_t M, int d, const T* g1, const T* b1,
                          const T* g2, const T* b2, float eps, T* out1, T* out2) {
-  pdl_trigger();
   extern __shared__ __align__(16) uint8_t smem_few[];
   T* sp = reinterpret_cast<T*>(smem_few);
   stage_norm_params(g1, RMS ? nullptr : b1, out2 ? g2 : nullptr, (RMS || !out2) ? nullptr : b2, d, sp);
   pdl_wait();
+  pdl_trigger();
   const int64_t lo = (int64_t)blockIdx.x * kFewRowWarps;
   const int64_t hi = lo + kFewRowWarps < M ? lo + kFewRowWarps : M;
   norm_share<T, RMS, NCH>(
@@ -211,11 +211,11 @@ __global__ void __launch_bounds__(32 * kFewRowWarps)
     decide_norm_kernel(const T* x, int B, int d, const T* g1, const T* b1, const T* g2, const T* b2, float eps,
                        T* out1, T* out2, const float* scores, const float* thr, const int32_t* hdr, int C_max,
                        int32_t* rows, int32_t* pos, int32_t* kept_out, int* err) {
-  pdl_trigger();
   extern __shared__ __align__(16) uint8_t smem_dn[];
   T* sp = reinterpret_cast<T*>(smem_dn);
   stage_norm_params(g1, RMS ? nullptr : b1, out2 ? g2 : nullptr, (RMS || !out2) ? nullptr : b2, d, sp);
   pdl_wait();
+  pdl_trigger();
   const int64_t lo = (int64_t)blockIdx.x * kFewRowWarps;
   const int64_t hi = lo + kFewRowWarps < B ? lo + kFewRowWarps : B;
   const int b = (int)lo + (int)(threadIdx.x >> 5);
@@ -277,7 +277,6 @@ __global__ void __launch_bounds__(kRowThreads)
     gather_norm_tma_kernel(const T* x, const int32_t* rows, int64_t M, int d, const T* g1,
                            const T* b1, const T* g2, const T* b2, float eps, T* out1, T* out2,
                            int* err, unsigned long long timeout_ns) {
-  pdl_trigger();
   extern __shared__ __align__(16) uint8_t smem_rows[];
   constexpr int V = Elem<T>::kVec;
   const uint32_t row_bytes = (uint32_t)d * sizeof(T);
@@ -298,6 +297,7 @@ __global__ void __launch_bounds__(kRowThreads)
   stage_norm_params(g1, RMS ? nullptr : b1, out2 ? g2 : nullptr, (RMS || !out2) ? nullptr : b2, d,
                     sp);   // weights: independent of the previous kernel (also syncs the block)
   pdl_wait();
+  pdl_trigger();
   const int64_t lo = (int64_t)blockIdx.x * M / gridDim.x, hi = (int64_t)(blockIdx.x + 1) * M / gridDim.x;
   const int64_t n = hi - lo;
   volatile int* abort_v = &abort_flag;
@@ -426,8 +426,8 @@ struct InvFreq {
   double v[64];
 };
 __global__ void rope_table_kernel(float2* tab, int T, int half, InvFreq inv) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= (int64_t)T * half) return;
   const int p = (int)(k / half), i = (int)(k % half);
@@ -444,8 +444,8 @@ __global__ void rope_table_kernel(float2* tab, int T, int half, InvFreq inv) {
 template <typename T>
 __global__ void rope_apply_kernel(T* qkv, int64_t M, int64_t ld, int heads, int head_dim,
                                   int half, const int32_t* pos, int seq_len, const float2* tab) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t per_row = (int64_t)heads * half;
   if (k >= M * per_row) return;
@@ -469,8 +469,8 @@ __global__ void rope_apply_kernel(T* qkv, int64_t M, int64_t ld, int heads, int 
 __global__ void __launch_bounds__(kRrThreads, 2)
     router_f32_kernel(const float* x, int64_t n, int d, int h, const float* w1, const float* b1, const float* w2,
                       const float* b2, float* scores) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   extern __shared__ __align__(16) float smem_rr[];
   const int lane = threadIdx.x & 31;
   const int64_t r0 = (int64_t)blockIdx.x * kRrRows;
@@ -501,8 +501,8 @@ constexpr int kTopkThreads = 1024;
 // One block per sequence: idx[b][i] = i-th kept position (ascending), rows[b][i] = b T + position.
 __global__ void __launch_bounds__(kTopkThreads) topk_kernel(const float* scores, int T, int K,
                                                             int32_t* idx, int32_t* rows) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   extern __shared__ uint32_t keys[];
   __shared__ TopkShared sh;
   const int b = blockIdx.x;
@@ -529,7 +529,6 @@ __global__ void __launch_bounds__(kSelThreads)
     select_gather_norm_kernel(const float* scores, int Tlen, int K, const T* x, int d, const T* g1,
                               const T* b1, const T* g2, const T* b2, float eps, T* out1, T* out2,
                               int32_t* idx, int32_t* rows) {
-  pdl_trigger();
   extern __shared__ __align__(16) uint32_t smem_sel[];
   T* sp = reinterpret_cast<T*>(smem_sel);                               // [4][d] norm parameters
   uint32_t* keys = smem_sel + (4 * d * sizeof(T)) / 4;                  // [Tlen]
@@ -538,6 +537,7 @@ __global__ void __launch_bounds__(kSelThreads)
   stage_norm_params(g1, RMS ? nullptr : b1, out2 ? g2 : nullptr, (RMS || !out2) ? nullptr : b2, d,
                     sp);   // weights: independent of the previous kernel
   pdl_wait();
+  pdl_trigger();
   const int b = blockIdx.y, g = blockIdx.x, G = gridDim.x;
   const float* sc = scores + (int64_t)b * Tlen;
   for (int t = threadIdx.x; t < Tlen; t += kSelThreads) keys[t] = score_key(sc[t]);
@@ -567,8 +567,8 @@ template <typename T>
 __global__ void __launch_bounds__(kStatThreads) cos_rows_kernel(const T* a, const T* b,
                                                                 int64_t n_rows, int d, int mode,
                                                                 double* partials) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   constexpr int V = Elem<T>::kVec;
   __shared__ double red[kStatThreads / 32][3];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -612,8 +612,8 @@ __global__ void __launch_bounds__(kStatThreads) cos_rows_kernel(const T* a, cons
 // cos_rows_kernel.
 __global__ void __launch_bounds__(kStatThreads) cos_chunks_kernel(const float4* parts, int64_t n_rows,
                                                                   int nch, int mode, double* partials) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ double red[kStatThreads / 32][3];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t nwarps = (int64_t)gridDim.x * (kStatThreads / 32);
@@ -648,8 +648,8 @@ __global__ void __launch_bounds__(kStatThreads) cos_chunks_kernel(const float4* 
 // Fixed-order sum of the per-block partials, added to acc.
 __global__ void cos_finish_kernel(const double* partials, int nblocks, int64_t n_rows, int mode,
                                   double* acc) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ double red[3][256];
   double s[3] = {0, 0, 0};
   for (int i = threadIdx.x; i < nblocks; i += 256)
@@ -679,8 +679,8 @@ static __device__ __align__(256) double g_stats_scratch[kStatMaxBlocks * 3];
 
 // idx[b * K + j] = j: the kept positions of a dense layer.
 __global__ void iota_kernel(int32_t* idx, int64_t n, int K) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k < n) idx[k] = (int32_t)(k % K);
 }

@@ -23,8 +23,8 @@ int row_blocks(int64_t n) {
 
 // Fixed-order sum of one double per block, added to acc[0]; acc[1] += count.
 __global__ void sum_partials_kernel(const double* partials, int nblocks, int64_t count, double* acc) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ double red[256];
   double s = 0;
   for (int i = threadIdx.x; i < nblocks; i += 256) s += partials[i];
@@ -61,8 +61,8 @@ __device__ __forceinline__ void block_partial(double mine, double* partials) {
 template <typename T>
 __global__ void __launch_bounds__(kRowThreadsT)
     align_hidden_kernel(const T* hs, const T* hd, int64_t n_rows, int d, float* grad, double* partials) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
   const int64_t nw = (int64_t)gridDim.x * (kRowThreadsT / 32);
   double mine = 0;
@@ -122,8 +122,8 @@ constexpr int kAlignThreads = 512;
 template <typename T, int G, int NV>
 __global__ void __launch_bounds__(kAlignThreads)
     align_hidden_vec_kernel(const T* hs, const T* hd, int64_t n_rows, int d, float* grad, double* partials) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   constexpr int V = Elem<T>::kVec, GROUPS = kAlignThreads / G, W = G / 32;
   __shared__ float2 xch[3][GROUPS][W];
   const int grp = threadIdx.x / G, gt = threadIdx.x % G;
@@ -225,8 +225,8 @@ __global__ void __launch_bounds__(kAlignThreads)
 // sums where they are computed, kl_tc.cu).
 __global__ void __launch_bounds__(kRowThreadsT)
     kl_rows_kernel(const float* ls, const float* ld, int64_t n_rows, int n_cls, double* partials) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
   const int64_t nw = (int64_t)gridDim.x * (kRowThreadsT / 32);
   double mine = 0;
@@ -272,8 +272,8 @@ __global__ void __launch_bounds__(kRrThreads, 2)
     router_bwd_rows_kernel(const T* x, const T* y_plain, const int32_t* rows, int64_t M, int d, int h,
                            const T* w1, const T* b1, const T* w2, const T* b2, const float* G, int vec, float* du,
                            float* su, float* ds_out) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   extern __shared__ __align__(16) float smem_rr[];
   __shared__ float gd_s[kRrRows];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -356,8 +356,8 @@ template <typename T>
 __global__ void __launch_bounds__(kRedThreads)
     router_bwd_reduce_kernel(const T* x, const int32_t* rows, int64_t M, int d, int h, const float* du,
                              const float* su, const float* ds, float* grad) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   constexpr int V = Elem<T>::kVec;
   constexpr int XV = kRedRows * kRedCols / V / kRedThreads;   // 16-byte x vectors a thread
   __shared__ __align__(16) float sdu[kRedRows][64];
