@@ -483,8 +483,8 @@ typedef enum {
   ADADSF_KERNEL_ATTENTION, ADADSF_KERNEL_GEMM_O, ADADSF_KERNEL_NORM2, ADADSF_KERNEL_GEMM_UP,
   ADADSF_KERNEL_GEMM_DOWN, ADADSF_KERNEL_STATS, ADADSF_KERNEL_FINAL_NORM, ADADSF_KERNEL_COPY,
   ADADSF_KERNEL_LINEAR, ADADSF_KERNEL_SELFTEST,
-  ADADSF_KERNEL_GEMM_QKV_UP,   /* GPT-NeoX, bf16: QKV and MLP-up projections in one launch */
-  ADADSF_KERNEL_GEMM_O_DOWN,   /* GPT-NeoX, bf16: output + MLP-down projections, one accumulator */
+  ADADSF_KERNEL_GEMM_QKV_UP,   /* GPT-NeoX: QKV and MLP-up projections in one launch */
+  ADADSF_KERNEL_GEMM_O_DOWN,   /* GPT-NeoX: output + MLP-down projections, one accumulator */
   ADADSF_KERNEL_TOPK_GATHER_NORM, /* Top-K fused with the gather and norms of the kept rows */
   ADADSF_KERNEL_DECIDE,        /* decode: keep decision of each new token (inside the norm launch when the step runs on one stream) */
   ADADSF_KERNEL_KV_CACHE,      /* decode cache: fill (prefill), thresholds, append */

@@ -465,15 +465,15 @@ adadsf_status layer_impl(const adadsf_model_cfg* c, const adadsf_layer_weights* 
                     "norm")));
   }
   // a5: QKV projection (+bias), rotary at the original positions.
-  // On the tensor-core path the rotation is fused into the QKV epilogue, and
-  // for GPT-NeoX (parallel residual) the MLP up projection of the second
-  // norm shares the launch (a8).
+  // The rotation is fused into the QKV epilogue where the kernel can, and for
+  // GPT-NeoX (parallel residual) the MLP up projection of the second norm
+  // shares the launch (a8).
   const int half = c->rotary_dim / 2;
   // (not in a decode step: with a few rows the projection runs split along K,
   // which rotary tiles of halves above 16 features rule out; a separate pass
   // rotates the few rows instead)
-  const bool fuse_rope = tc && !dec && (half == 4 || half == 8 || half == 16 || (half > 0 && half % 32 == 0));
-  const bool neox_tc = neox && tc;
+  const bool fuse_rope = !dec && (tc ? half == 4 || half == 8 || half == 16 || (half > 0 && half % 32 == 0)
+                                     : f32_fuses_rope(half, c->head_dim));
   {
     GemmArgs g = linear_args(fuse1 ? x : lb.n1, d, w->w_qkv, M, qkv_dim, d);
     g.scratch = lb.split;
@@ -506,7 +506,7 @@ adadsf_status layer_impl(const adadsf_model_cfg* c, const adadsf_layer_weights* 
       g.epi.vt_hd = c->head_dim;
       g.epi.vt_hkv = c->n_kv_heads;
     }
-    if (neox_tc) {
+    if (neox) {
       // act = GELU(LN2 x W_up^T + b_up), grouped with the QKV tiles (first:
       // its GELU epilogue is the costlier)
       GemmArgs u = linear_args(lb.n2, d, w->w_up, M, F, d);
@@ -514,9 +514,9 @@ adadsf_status layer_impl(const adadsf_model_cfg* c, const adadsf_layer_weights* 
       u.epi.act = ACT_GELU;
       u.epi.out = lb.act;
       u.epi.ld_out = F;
-      TRY(launch(dev, ADADSF_KERNEL_GEMM_QKV_UP, true, 2.0 * M * ((double)qkv_dim + F) * d,
+      TRY(launch(dev, ADADSF_KERNEL_GEMM_QKV_UP, tc, 2.0 * M * ((double)qkv_dim + F) * d,
                  (2.0 * Md + ((double)qkv_dim + F) * d + (double)M * (qkv_dim + F)) * es,
-                 CALL(gemm_bf16_grouped(u, g, dev), "qkv + mlp up projections")));
+                 CALL(tc ? gemm_bf16_grouped(u, g, dev) : gemm_f32_grouped(u, g, dev), "qkv + mlp up projections")));
     } else {
       TRY(launch(dev, ADADSF_KERNEL_GEMM_QKV, tc, 2.0 * M * qkv_dim * d,
                  (Md + (double)qkv_dim * d + (double)M * qkv_dim) * es,
@@ -563,7 +563,7 @@ adadsf_status layer_impl(const adadsf_model_cfg* c, const adadsf_layer_weights* 
     TRY(launch(dev, ADADSF_KERNEL_KV_CACHE, false, 0, 8.0 * M,
                CALL(kv_threshold(lb.scores, lb.idx, B, T, K, sink->lens, sink->thr, dev), "cache thresholds")));
   }
-  if (neox_tc) {
+  if (neox) {
     // a7 + a8 + a9 as one GEMM with two K sources (parallel residual, Eq. 2):
     // x[row] = x[row] + O W_o^T + act W_down^T + b_o + b_down
     GemmArgs g = linear_args(lb.attn, q, w->w_o, M, d, q);
@@ -588,44 +588,9 @@ adadsf_status layer_impl(const adadsf_model_cfg* c, const adadsf_layer_weights* 
       g.epi.cos_out = lb.cospart;
       g.epi.cos_ld = d / 32;
     }
-    TRY(launch(dev, ADADSF_KERNEL_GEMM_O_DOWN, true, 2.0 * M * d * ((double)q + F),
+    TRY(launch(dev, ADADSF_KERNEL_GEMM_O_DOWN, tc, 2.0 * M * d * ((double)q + F),
                ((double)M * (q + F) + (double)d * (q + F) + 2.0 * Md) * es,
                [&] { return run_linear(dt, g, dev, "output + mlp down projections + residual scatter"); }));
-  } else if (neox) {
-    // a7: attn_out = O W_o^T + b_o (packed)
-    GemmArgs g = linear_args(lb.attn, q, w->w_o, M, d, q);
-    g.scratch = lb.split;
-    g.scratch_bytes = lb.split ? gemm_split_scratch_bytes() : 0;
-    g.epi.bias = w->b_o;
-    g.epi.out = lb.ao;
-    g.epi.ld_out = d;
-    TRY(launch(dev, ADADSF_KERNEL_GEMM_O, tc, 2.0 * M * d * q, ((double)M * q + (double)d * q + Md) * es,
-               [&] { return run_linear(dt, g, dev, "output projection"); }));
-    // a8: act = GELU(LN2 x W_up^T + b_up)
-    GemmArgs u = linear_args(lb.n2, d, w->w_up, M, F, d);
-    u.epi.bias = w->b_up;
-    u.epi.act = ACT_GELU;
-    u.epi.out = lb.act;
-    u.epi.ld_out = F;
-    TRY(launch(dev, ADADSF_KERNEL_GEMM_UP, tc, 2.0 * M * F * d, (Md + (double)F * d + (double)M * F) * es,
-               [&] { return run_linear(dt, u, dev, "mlp up"); }));
-    // a8 + a9: x[row] = x[row] + attn_out + act W_down^T + b_down
-    GemmArgs dn = linear_args(lb.act, F, w->w_down, M, d, F);
-    dn.scratch = lb.split;
-    dn.scratch_bytes = lb.split ? gemm_split_scratch_bytes() : 0;
-    dn.epi.bias = w->b_down;
-    dn.epi.add_packed = lb.ao;
-    dn.epi.ld_add_packed = d;
-    dn.epi.add_rows = x;
-    dn.epi.ld_add_rows = d;
-    dn.epi.rows = rows;
-    dn.epi.out_mapped = true;
-    dn.epi.out = x;
-    dn.epi.ld_out = d;
-    if (gate) dn.epi.gate_scores = lb.scores;   // x[row] + sigmoid(s) delta
-    TRY(launch(dev, ADADSF_KERNEL_GEMM_DOWN, tc, 2.0 * M * d * F,
-               ((double)M * F + (double)d * F + 3.0 * Md) * es,
-               [&] { return run_linear(dt, dn, dev, "mlp down + residual scatter"); }));
   } else {
     // a7: h = x[row] + O W_o^T (packed)
     GemmArgs g = linear_args(lb.attn, q, w->w_o, M, d, q);

@@ -85,7 +85,6 @@ __global__ void __launch_bounds__(kAtThreads) attn_f32_kernel(const float* qkv, 
   };
   const int64_t kc0 = (int64_t)n_heads * HD + (int64_t)g * HD, vc0 = kc0 + (int64_t)n_kv * HD;
   pdl_wait();
-  pdl_trigger();
   load_rows(sQ, C::LD, (int64_t)h * HD, q0);
   load_rows(sK, C::LD, kc0, 0);
   load_rows(sV, HD, vc0, 0);
@@ -181,6 +180,7 @@ __global__ void __launch_bounds__(kAtThreads) attn_f32_kernel(const float* qkv, 
     }
     asm volatile("cp.async.wait_group 1;" ::: "memory");   // V of this tile
     __syncthreads();                                        // V has landed for all; P is the warp's own
+    if (diag) pdl_trigger();
     if (diag) pv(std::true_type());
     else pv(std::false_type());
     __syncthreads();   // V is read

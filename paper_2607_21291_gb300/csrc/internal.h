@@ -29,7 +29,7 @@ enum Act : int { ACT_NONE = 0, ACT_GELU = 1, ACT_SWIGLU = 2 };
 struct Epilogue {
   int act = ACT_NONE;
   const void* bias = nullptr;
-  const void* bias2 = nullptr;   // bf16 tensor-core path only
+  const void* bias2 = nullptr;
   const void* add_packed = nullptr;
   int64_t ld_add_packed = 0;
   const void* add_rows = nullptr;
@@ -39,9 +39,10 @@ struct Epilogue {
   void* out = nullptr;
   int64_t ld_out = 0;
   // Rotary embedding of the first rope_cols output columns (query and key
-  // heads), bf16 tensor-core path only: per head of rope_hd columns, feature
+  // heads): per head of rope_hd columns, feature
   // i < rope_half pairs with i + rope_half and turns by tab[pos][i], pos =
-  // rope_pos ? rope_pos[m] : m % rope_T. Needs rope_half in {4, 8, 16} or a multiple of 32.
+  // rope_pos ? rope_pos[m] : m % rope_T. bf16 needs rope_half in {4, 8, 16} or a
+  // multiple of 32; fp32 see f32_fuses_rope.
   const float2* rope_tab = nullptr;
   const int32_t* rope_pos = nullptr;
   int rope_T = 1, rope_half = 0, rope_hd = 0, rope_cols = 0;
@@ -77,8 +78,8 @@ struct Epilogue {
   int64_t ld_cos_in = 0;
 };
 
-// acc = A . W^T (+ A2 . Wk2^T when K2 > 0: a second K source, bf16
-// tensor-core path only, K a multiple of 64).
+// acc = A . W^T (+ A2 . Wk2^T when K2 > 0: a second K source, K a multiple of
+// 64 on the bf16 path and of 32 on the fp32 path).
 struct GemmArgs {
   const void* A = nullptr;  int64_t lda = 0;   // [M, K]
   const void* W = nullptr;  int64_t ldw = 0;   // [N, K]
@@ -142,6 +143,10 @@ cudaError_t kl_tc(const void* hs, const void* hd, const void* w, int64_t n_rows,
                   double* partials, double* acc, const Dev& dev);
 // gemm_simt.cu -- fp32 projections on CUDA cores.
 cudaError_t gemm_f32(const GemmArgs& a, const Dev& dev);
+// Two independent projections of the same K (no SwiGLU) in one launch.
+cudaError_t gemm_f32_grouped(const GemmArgs& a, const GemmArgs& b, const Dev& dev);
+// Whether gemm_f32 can rotate (rope_tab) heads of hd features with this many pairs.
+bool f32_fuses_rope(int half, int hd);
 
 // attention.cu -- causal attention among kept tokens, fp32 storage.
 cudaError_t attention(int dtype, const void* qkv, int64_t ld_qkv, void* out, int64_t ld_out, int B,

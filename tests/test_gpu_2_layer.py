@@ -305,3 +305,24 @@ def test_model_qwen_calibration_statistics(A):
                                       stats_mode="token")
     s_ref = np.array([O.similarity(a) for a in st])
     assert np.max(np.abs(A.adadsf_similarity(accs[0]) - s_ref)) < 5e-3
+
+
+@pytest.mark.parametrize("hd,rot,T,K,gated", [(128, 32, 150, 67, False), (64, 8, 90, 90, True), (64, 12, 70, 33, False),
+                                              (64, 64, 130, 129, True), (128, 0, 40, 20, False)])
+def test_layer_f32_rotary(A, hd, rot, T, K, gated):
+    """fp32 GPT-NeoX layers (QKV and MLP-up in one launch, output and MLP-down
+    in one sum) at rotary widths that the QKV epilogue rotates (whole groups of
+    four pairs, both halves in 32 columns) and that take the separate pass."""
+    shape = S.PYTHIA_70M.replace(n_layers=1, d=256, n_heads=256 // hd, n_kv_heads=256 // hd, head_dim=hd, ffn=320,
+                                 rotary_dim=rot)
+    W = H.host_layer(shape, hd + rot)
+    x = S.hidden(hd, 2, T, shape.d)
+    cfg = A.make_cfg(shape, A.FLAG_GATE_SIGMOID if gated else 0)
+    xd = H.to_dev(x, torch.float32)
+    idx = torch.empty((2, K), dtype=torch.int32, device="cuda")
+    ws = A.workspace(A.adadsf_layer_workspace_size(cfg, 2, T, K))
+    A.adadsf_sparse_layer_forward(cfg, A.to_device(W, torch.float32), xd, K, idx, None, ws)
+    assert A.adadsf_sync_check(ws) == A.OK
+    p = dict(O.params_of(shape), gate="sigmoid") if gated else O.params_of(shape)
+    ref, _, _ = O.sparse_layer_forward(x.astype(np.float64), H.f64(W), p, K, idx=idx.cpu().numpy())
+    H.assert_close(xd.cpu().numpy(), ref, H.F32_TOL, "fp32 layer")
