@@ -265,8 +265,9 @@ __global__ void __launch_bounds__(kRowThreadsT)
 // rows[m]): u = W1 x_r + b1 (h <= 64 hidden units, router_rows.cuh), s = w2 .
 // SiLU(u) + b2, the gate's ds = sigmoid'(s) (G_r . delta_r) with delta_r =
 // y_plain_r - x_r, and du = ds w2 SiLU'(u). Writes du [m][h], SiLU(u) [m][h]
-// and ds [m]. FFMA bound (the products stay exact and the sums fp32):
-// 2 M h d operations. G may be 4-byte aligned only (vec: 16-byte loads).
+// and ds [m]. bf16 (h = 64): u on warp-level tensor products, so the rows of x,
+// y_plain and G bound it; fp32: on FFMA. G may be 4-byte aligned only (vec: 16-byte
+// loads).
 template <typename T>
 __global__ void __launch_bounds__(kRrThreads, 2)
     router_bwd_rows_kernel(const T* x, const T* y_plain, const int32_t* rows, int64_t M, int d, int h,
@@ -305,8 +306,12 @@ __global__ void __launch_bounds__(kRrThreads, 2)
   }
   const int64_t ma = m0 + (lane >> 2) < M ? m0 + (lane >> 2) : M - 1;
   const int64_t mb = m0 + (lane >> 2) + 8 < M ? m0 + (lane >> 2) + 8 : M - 1;
-  const float4 u4 = router_rows_units<T>(x + (int64_t)rows[ma] * d, x + (int64_t)rows[mb] * d, w1, 0, h, d,
-                                         smem_rr);   // its barriers make gd_s visible
+  // its barriers make gd_s visible
+  float4 u4;
+  if constexpr (sizeof(T) == 2)
+    u4 = router_rows_units_mma(x + (int64_t)rows[ma] * d, x + (int64_t)rows[mb] * d, w1, d, smem_rr);
+  else
+    u4 = router_rows_units<T>(x + (int64_t)rows[ma] * d, x + (int64_t)rows[mb] * d, w1, 0, h, d, smem_rr);
   const int row = threadIdx.x >> 4, j0 = (threadIdx.x & 15) * 4;
   const float uu[4] = {u4.x, u4.y, u4.z, u4.w};
   float si[4], dsi[4], s = 0.f;
@@ -338,15 +343,33 @@ __global__ void __launch_bounds__(kRrThreads, 2)
 
 // Router gradient, part 2: dW1[j][k] = sum_m du[m][j] x[rows[m]][k]. A cluster
 // of 8 CTAs owns 64 columns k and all h <= 64 units; each CTA sums an eighth
-// of the rows in fp32 (8 units x 4 columns a thread, rows staged 32 at a time
-// with the next 32 in flight) and the eighths are added in rank order through
-// distributed shared memory. The split along m is what fills the GPU: the
-// output has only d / 64 such tiles (32 at d = 2048). The last cluster
-// sums db1[j] = sum_m du[m][j], dw2[j] = sum_m ds[m] SiLU(u)[m][j] and db2 =
-// sum_m ds[m] the same way. With part 1 it takes 76 us at M = 2048, d = 2048
-// (bf16) and 0.97 ms at M = 32768, against 1024 us and 20.8 ms for one warp a
-// row with 64 serial dots and a reduction of 17 blocks that summed the vectors
-// in one thread each.
+// of the rows (rows staged 32 at a time with the next 32 in flight) and the
+// eighths are added in rank order through distributed shared memory. The split
+// along m is what fills the GPU: the output has only d / 64 such tiles (32 at d =
+// 2048). fp32 x: 8 units x 4 columns a thread on FFMA. bf16 x: tensor products with
+// du cut into three bf16 parts that add up to it exactly (8 of its 24 bits each), the
+// smallest first, each 16 rows summed from zero and added in fp32, so nothing of
+// du's precision is lost. The last cluster sums db1[j] = sum_m du[m][j], dw2[j] = sum_m
+// ds[m] SiLU(u)[m][j] and db2 = sum_m ds[m] the same way. With part 1 it takes
+// 29 us at M = 2048, d = 2048 (bf16) and 0.42 ms at M = 32768; 76 us and 0.97
+// ms with both parts on FFMA, 1024 us and 20.8 ms for one warp a row with 64 serial
+// dots and a reduction of 17 blocks that summed the vectors in one thread each.
+__device__ __forceinline__ void ldsm_x4_trans(uint32_t addr, uint32_t (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+// f as a sum of three bf16 values (in the high halves of p): exact for finite f
+// (each part takes the next 8 significant bits), f itself rounded where it is not.
+__device__ __forceinline__ void bf16_parts(float f, uint32_t (&p)[3]) {
+  const bool finite = fabsf(f) <= 3.402823466e38f;
+  p[0] = finite ? __float_as_uint(f) & 0xffff0000u : (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(f)) << 16;
+  const float r = f - __uint_as_float(p[0]);
+  p[1] = finite ? __float_as_uint(r) & 0xffff0000u : 0u;
+  p[2] = finite ? __float_as_uint(r - __uint_as_float(p[1])) & 0xffff0000u : 0u;
+}
+
 constexpr int kRedCluster = 8;
 constexpr int kRedThreads = 128;
 constexpr int kRedCols = 64;
@@ -360,8 +383,11 @@ __global__ void __launch_bounds__(kRedThreads)
   pdl_trigger();
   constexpr int V = Elem<T>::kVec;
   constexpr int XV = kRedRows * kRedCols / V / kRedThreads;   // 16-byte x vectors a thread
-  __shared__ __align__(16) float sdu[kRedRows][64];
-  __shared__ __align__(16) float sx[kRedRows][kRedCols];
+  constexpr bool MMA = sizeof(T) == 2;
+  __shared__ __align__(16) float sdu[MMA ? 1 : kRedRows][64];
+  __shared__ __align__(16) float sx[MMA ? 1 : kRedRows][kRedCols];
+  // MMA: rows of 64 bf16, 16-byte chunks XOR-ed with row % 8; three parts of du, x
+  __shared__ __align__(16) uint8_t sb[MMA ? 4 : 1][MMA ? kRedRows * 128 : 16];
   __shared__ __align__(16) float part[64 * kRedCols];
   const int rank = (int)cluster_ctarank();
   const int col0 = (int)(blockIdx.x / kRedCluster) * kRedCols;
@@ -399,62 +425,145 @@ __global__ void __launch_bounds__(kRedThreads)
     cluster_sync();   // the partials stay until every CTA has read them
     return;
   }
-  const int ty = tid >> 4, tx = tid & 15;   // units 8 ty .. + 7, columns 4 tx .. + 3
-  float acc[8][4];
+  const int ty = tid >> 4, tx = tid & 15;   // FFMA: units 8 ty .. + 7, columns 4 tx .. + 3
+  if constexpr (MMA) {
+    const int lane = tid & 31, warp = tid >> 5;
+    const int u0 = (warp >> 1) * 32, c0 = (warp & 1) * 32;   // the warp's 32 units x 32 columns
+    float tot[2][4][4];
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) acc[i][c] = 0.f;
-  float dv[kRedRows * 64 / kRedThreads];
-  uint4 xv[XV];
-  auto fetch = [&](int64_t m0) {
+      for (int j = 0; j < 4; ++j) tot[i][j][0] = tot[i][j][1] = tot[i][j][2] = tot[i][j][3] = 0.f;
+    float2 dv[kRedRows / 4];
+    uint4 xv[2];
+    auto fetch = [&](int64_t m0) {
 #pragma unroll
-    for (int i = 0; i < kRedRows * 64 / kRedThreads; ++i) {
-      const int mm = i * (kRedThreads / 64) + (tid >> 6), jj = tid & 63;
-      dv[i] = (m0 + mm < m_hi && jj < h) ? du[(m0 + mm) * h + jj] : 0.f;
+      for (int i = 0; i < kRedRows / 4; ++i) {   // rows warp + 4 i, units 2 lane and + 1
+        const int64_t m = m0 + warp + 4 * i;
+        dv[i] = m < m_hi ? *reinterpret_cast<const float2*>(du + m * h + 2 * lane) : make_float2(0.f, 0.f);
+      }
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int64_t m = m0 + (tid >> 3) + 16 * i;
+        xv[i] = m < m_hi ? *reinterpret_cast<const uint4*>(x + (int64_t)rows[m] * d + col0 + (tid & 7) * 8)
+                         : make_uint4(0, 0, 0, 0);
+      }
+    };
+    const uint32_t sbase = smem_u32(&sb[0][0]);
+    constexpr uint32_t PLANE = kRedRows * 128;
+    if (m_lo < m_hi) fetch(m_lo);
+    for (int64_t m0 = m_lo; m0 < m_hi; m0 += kRedRows) {
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < kRedRows / 4; ++i) {
+        const int r = warp + 4 * i;
+        uint32_t p0[3], p1[3];
+        bf16_parts(dv[i].x, p0);
+        bf16_parts(dv[i].y, p1);
+        const uint32_t off = r * 128 + ((((uint32_t)lane >> 2) ^ (r & 7)) << 4) + (lane & 3) * 4;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) *reinterpret_cast<uint32_t*>(&sb[k][off]) = (p0[k] >> 16) | (p1[k] & 0xffff0000u);
+      }
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int r = (tid >> 3) + 16 * i;
+        *reinterpret_cast<uint4*>(&sb[3][r * 128 + (((tid & 7) ^ (r & 7)) << 4)]) = xv[i];
+      }
+      __syncthreads();
+      if (m0 + kRedRows < m_hi) fetch(m0 + kRedRows);
+      const int mi = lane >> 3, mr = lane & 7;   // ldmatrix: this lane's matrix and row
+#pragma unroll
+      for (int ks = 0; ks < kRedRows; ks += 16) {
+        uint32_t b[2][4];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {   // columns c0 + 16 q: rows ks + 8 (mi & 1), column chunk mi / 2
+          const int r = ks + (mi & 1) * 8 + mr, c = (c0 >> 3) + 2 * q + (mi >> 1);
+          ldsm_x4_trans(sbase + 3 * PLANE + r * 128 + ((c ^ (r & 7)) << 4), b[q]);
+        }
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt) {
+          uint32_t a[3][4];
+          const int r = ks + (mi >> 1) * 8 + mr, c = (u0 >> 3) + 2 * mt + (mi & 1);
+#pragma unroll
+          for (int k = 0; k < 3; ++k) ldsm_x4_trans(sbase + k * PLANE + r * 128 + ((c ^ (r & 7)) << 4), a[k]);
+#pragma unroll
+          for (int nt = 0; nt < 4; ++nt) {
+            float p[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int k = 2; k >= 0; --k)
+              mma_16816(p, a[k][0], a[k][1], a[k][2], a[k][3], b[nt >> 1][(nt & 1) * 2], b[nt >> 1][(nt & 1) * 2 + 1]);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) tot[mt][nt][e] += p[e];
+          }
+        }
+      }
     }
+    const int gid = lane >> 2, tig = lane & 3;
 #pragma unroll
-    for (int i = 0; i < XV; ++i) {
-      const int v = i * kRedThreads + tid;
-      const int64_t m = m0 + v / (kRedCols / V);
-      xv[i] = m < m_hi ? *reinterpret_cast<const uint4*>(x + (int64_t)rows[m] * d + col0 + (v % (kRedCols / V)) * V)
-                       : make_uint4(0, 0, 0, 0);
-    }
-  };
-  if (m_lo < m_hi) fetch(m_lo);
-  for (int64_t m0 = m_lo; m0 < m_hi; m0 += kRedRows) {
-    __syncthreads();
+    for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-    for (int i = 0; i < kRedRows * 64 / kRedThreads; ++i) sdu[i * (kRedThreads / 64) + (tid >> 6)][tid & 63] = dv[i];
+      for (int nt = 0; nt < 4; ++nt) {
+        float* q = part + (u0 + 16 * mt + gid) * kRedCols + c0 + 8 * nt + 2 * tig;
+        *reinterpret_cast<float2*>(q) = make_float2(tot[mt][nt][0], tot[mt][nt][1]);
+        *reinterpret_cast<float2*>(q + 8 * kRedCols) = make_float2(tot[mt][nt][2], tot[mt][nt][3]);
+      }
+  } else {
+    float acc[8][4];
 #pragma unroll
-    for (int i = 0; i < XV; ++i) {
-      const int v = i * kRedThreads + tid;
-      float f[V];
-      unpack16(xv[i], f, T());
-      float* p = &sx[v / (kRedCols / V)][(v % (kRedCols / V)) * V];
+    for (int i = 0; i < 8; ++i)
 #pragma unroll
-      for (int e = 0; e < V; e += 4) *reinterpret_cast<float4*>(p + e) = make_float4(f[e], f[e + 1], f[e + 2], f[e + 3]);
-    }
-    __syncthreads();
-    if (m0 + kRedRows < m_hi) fetch(m0 + kRedRows);
-    const int nm = (int)(m_hi - m0 < kRedRows ? m_hi - m0 : kRedRows);
+      for (int c = 0; c < 4; ++c) acc[i][c] = 0.f;
+    float dv[kRedRows * 64 / kRedThreads];
+    uint4 xv[XV];
+    auto fetch = [&](int64_t m0) {
+#pragma unroll
+      for (int i = 0; i < kRedRows * 64 / kRedThreads; ++i) {
+        const int mm = i * (kRedThreads / 64) + (tid >> 6), jj = tid & 63;
+        dv[i] = (m0 + mm < m_hi && jj < h) ? du[(m0 + mm) * h + jj] : 0.f;
+      }
+#pragma unroll
+      for (int i = 0; i < XV; ++i) {
+        const int v = i * kRedThreads + tid;
+        const int64_t m = m0 + v / (kRedCols / V);
+        xv[i] = m < m_hi ? *reinterpret_cast<const uint4*>(x + (int64_t)rows[m] * d + col0 + (v % (kRedCols / V)) * V)
+                         : make_uint4(0, 0, 0, 0);
+      }
+    };
+    if (m_lo < m_hi) fetch(m_lo);
+    for (int64_t m0 = m_lo; m0 < m_hi; m0 += kRedRows) {
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < kRedRows * 64 / kRedThreads; ++i) sdu[i * (kRedThreads / 64) + (tid >> 6)][tid & 63] = dv[i];
+#pragma unroll
+      for (int i = 0; i < XV; ++i) {
+        const int v = i * kRedThreads + tid;
+        float f[V];
+        unpack16(xv[i], f, T());
+        float* p = &sx[v / (kRedCols / V)][(v % (kRedCols / V)) * V];
+#pragma unroll
+        for (int e = 0; e < V; e += 4) *reinterpret_cast<float4*>(p + e) = make_float4(f[e], f[e + 1], f[e + 2], f[e + 3]);
+      }
+      __syncthreads();
+      if (m0 + kRedRows < m_hi) fetch(m0 + kRedRows);
+      const int nm = (int)(m_hi - m0 < kRedRows ? m_hi - m0 : kRedRows);
 #pragma unroll 4
-    for (int mm = 0; mm < nm; ++mm) {
-      const float4 a0 = *reinterpret_cast<const float4*>(&sdu[mm][8 * ty]);
-      const float4 a1 = *reinterpret_cast<const float4*>(&sdu[mm][8 * ty + 4]);
-      const float4 b = *reinterpret_cast<const float4*>(&sx[mm][4 * tx]);
-      const float af[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-      const float bf[4] = {b.x, b.y, b.z, b.w};
+      for (int mm = 0; mm < nm; ++mm) {
+        const float4 a0 = *reinterpret_cast<const float4*>(&sdu[mm][8 * ty]);
+        const float4 a1 = *reinterpret_cast<const float4*>(&sdu[mm][8 * ty + 4]);
+        const float4 b = *reinterpret_cast<const float4*>(&sx[mm][4 * tx]);
+        const float af[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+        const float bf[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
+        for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[i][c] = fmaf(af[i], bf[c], acc[i][c]);
+          for (int c = 0; c < 4; ++c) acc[i][c] = fmaf(af[i], bf[c], acc[i][c]);
+      }
     }
-  }
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
-    *reinterpret_cast<float4*>(part + (8 * ty + i) * kRedCols + 4 * tx) =
-        make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+    for (int i = 0; i < 8; ++i)
+      *reinterpret_cast<float4*>(part + (8 * ty + i) * kRedCols + 4 * tx) =
+          make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+  }
   cluster_sync();
   {
     // this CTA finishes units [8 rank, 8 rank + 8): one 16-byte piece a thread
@@ -480,10 +589,11 @@ cudaError_t router_backward_t(const void* x, const void* y_plain, const int32_t*
                               float* su, float* ds, float* grad, const Dev& dev) {
   const int64_t nb = (M + kRrRows - 1) / kRrRows;
   if (nb > INT32_MAX) return cudaErrorInvalidValue;
-  cudaError_t e = allow_smem(router_bwd_rows_kernel<T>, RouterRows<T>::SMEM_BYTES);
+  constexpr int smem = sizeof(T) == 2 ? RouterRows<T>::MMA_BYTES : RouterRows<T>::SMEM_BYTES;
+  cudaError_t e = allow_smem(router_bwd_rows_kernel<T>, smem);
   if (e != cudaSuccess) return e;
   const int vec = (reinterpret_cast<uintptr_t>(G) & 15u) == 0 ? 1 : 0;
-  e = launch_pdl(router_bwd_rows_kernel<T>, dim3((unsigned)nb), dim3(kRrThreads), RouterRows<T>::SMEM_BYTES, dev.stream,
+  e = launch_pdl(router_bwd_rows_kernel<T>, dim3((unsigned)nb), dim3(kRrThreads), smem, dev.stream,
                  static_cast<const T*>(x), static_cast<const T*>(y_plain), rows, M, d, h, static_cast<const T*>(w1),
                  static_cast<const T*>(b1), static_cast<const T*>(w2), static_cast<const T*>(b2), G, vec, du, su, ds);
   if (e != cudaSuccess) return e;
