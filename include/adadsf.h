@@ -487,7 +487,7 @@ typedef enum {
   ADADSF_KERNEL_GEMM_O_DOWN,   /* GPT-NeoX: output + MLP-down projections, one accumulator */
   ADADSF_KERNEL_TOPK_GATHER_NORM, /* Top-K fused with the gather and norms of the kept rows */
   ADADSF_KERNEL_DECIDE,        /* decode: keep decision of each new token (inside the norm launch when the step runs on one stream) */
-  ADADSF_KERNEL_KV_CACHE,      /* decode cache: fill (prefill), thresholds, append */
+  ADADSF_KERNEL_KV_CACHE,      /* decode cache: fill (prefill), thresholds */
   ADADSF_KERNEL_ALIGN,         /* alignment objective and router gradient (Eqs. 9-10) */
   ADADSF_KERNEL_COUNT
 } adadsf_kernel_kind;

@@ -413,7 +413,7 @@ adadsf_status layer_impl(const adadsf_model_cfg* c, const adadsf_layer_weights* 
     // projections stream their weights once either way)
     if (forked) {
       TRY(launch(sdev, ADADSF_KERNEL_DECIDE, false, 0, 16.0 * B,
-                 CALL(decode_decide(lb.scores, dec->thr, dec->hdr, B, dec->C_max, dec->rows, dec->pos,
+                 CALL(decode_decide(lb.scores, dec->thr, dec->hdr, B, dec->C_max, dec->lens, dec->rows, dec->pos,
                                     dec->kept_out, sdev),
                       "keep decision")));
       CUDA_TRY(cudaEventRecord(dec->join, dec->side), "join the router stream");
@@ -425,7 +425,7 @@ adadsf_status layer_impl(const adadsf_model_cfg* c, const adadsf_layer_weights* 
       TRY(launch(dev, ADADSF_KERNEL_GATHER_NORM, false, 0, Md * es * (neox ? 3 : 2) + 16.0 * B,
                  CALL(decide_norm(dt, x, B, d, !neox, w->ln1_w, w->ln1_b, w->ln2_w, w->ln2_b, c->norm_eps,
                                   lb.n1, neox ? lb.n2 : nullptr, lb.scores, dec->thr, dec->hdr, dec->C_max,
-                                  dec->rows, dec->pos, dec->kept_out, dev),
+                                  dec->lens, dec->rows, dec->pos, dec->kept_out, dev),
                       "keep decision + norm")));
     }
     rows = dec->rows;
@@ -531,20 +531,30 @@ adadsf_status layer_impl(const adadsf_model_cfg* c, const adadsf_layer_weights* 
                     "rotary")));
   if (dec) {
     if (forked) CUDA_TRY(cudaStreamWaitEvent(dev.stream, dec->join, 0), "join the router stream");
-    // a5' + a6 (decode): rotary of the new rows fused with the cache append
-    // (a kept token's rotated key and value join the cache), then each new
-    // token attends to its layer's cached kept tokens (itself included when kept)
-    TRY(launch(dev, ADADSF_KERNEL_KV_CACHE, false, 0,
-               2.0 * M * (c->n_heads + c->n_kv_heads) * c->rotary_dim * es + 4.0 * B * kv * es,
-               CALL(rope_append(dt, lb.qkv, qkv_dim, c->n_heads, c->n_kv_heads, c->head_dim, c->rotary_dim, B,
-                                dec->rows, dec->pos, lb.rope, dec->lens, dec->C_max, dec->kc, dec->vc, dev),
-                    "rotary + cache append")));
+    // a5' + a6 (decode): rotary of the new rows, the cache append (a kept token's
+    // rotated key and value join the cache), then each new token attends to its
+    // layer's cached kept tokens (itself included when kept)
+    DecodeAttn at_;
+    at_.qkv = lb.qkv;
+    at_.ld = qkv_dim;
+    at_.Hq = c->n_heads;
+    at_.Hkv = c->n_kv_heads;
+    at_.hd = c->head_dim;
+    at_.half = half;
+    at_.C_max = dec->C_max;
+    at_.B = B;
+    at_.kc = dec->kc;
+    at_.vc = dec->vc;
+    at_.lens = dec->lens;
+    at_.pos = dec->pos;
+    at_.tab = lb.rope;
+    at_.part_o = dec->part_o;
+    at_.part_ml = dec->part_ml;
+    at_.out = lb.attn;
+    at_.ld_out = q;
     TRY(launch(dev, ADADSF_KERNEL_ATTENTION, false, 0,
                (double)B * 2.0 * q * es + 2.0 * B * kv * es * dec->C_max,
-               CALL(decode_attention(dt, lb.qkv, qkv_dim, c->n_heads, c->n_kv_heads, c->head_dim, dec->kc,
-                                     dec->vc, dec->lens, dec->C_max, B, dec->part_o, dec->part_ml, lb.attn, q,
-                                     dev),
-                    "decode attention")));
+               CALL(decode_attention(dt, at_, dev), "decode attention")));
   } else {
     // a6: causal attention among the kept tokens.
     TRY(launch(dev, ADADSF_KERNEL_ATTENTION, tc, 2.0 * B * c->n_heads * c->head_dim * (double)K * (K + 1),

@@ -433,6 +433,30 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
          | ((uint32_t)(M >> 4) << 24); // M / 16
 }
 
+// Keep decision of sequence b's new token at one layer (see decode_decide_kernel).
+__device__ __forceinline__ void decide_row(int b, const float* scores, const float* thr, const int32_t* hdr, int C_max,
+                                           int32_t* lens, int32_t* rows, int32_t* pos, int32_t* kept_out, int* err) {
+  int t = hdr[0];
+  if (hdr[1] != C_max || t < 0 || t >= C_max) {
+    set_device_error(err, DEVERR_INDEX);
+    t = t < 0 ? 0 : (t >= C_max ? C_max - 1 : t);
+  }
+  const bool keep = scores[b] > thr[b];
+  bool append = keep;
+  if (keep) {
+    const int len = lens[b];
+    if (len < 0 || len >= C_max) {   // the layer's cache is full: nothing appended
+      set_device_error(err, DEVERR_INDEX);
+      append = false;
+    } else {
+      lens[b] = len + 1;
+    }
+  }
+  rows[b] = keep ? b : -1;
+  pos[b] = t | (append ? kDecAppend : 0);
+  if (kept_out) kept_out[b] = keep ? 1 : 0;
+}
+
 // Host: let `kernel` use `bytes` of dynamic shared memory on the current device.
 template <typename K>
 inline cudaError_t allow_smem(K kernel, int bytes) {

@@ -93,26 +93,20 @@ __global__ void cache_header_kernel(int32_t* hdr, int T, int C_max, int L, int B
 // ---------------------------------------------------------------- decode step
 // Keep decision of the new token of every sequence at one layer, its
 // position, and the packed-row map of the projections (rows[b] = b if kept,
-// -1 if it bypasses the layer: the residual scatter then skips it). A tie
+// -1 if it bypasses the layer: the residual scatter then skips it). A kept token
+// with room in the layer's cache is counted there at once (its key and value
+// follow before the step's attention) and bit kDecAppend of pos[b] says so. A tie
 // loses and NaN never wins. A cache not filled by a prefill of this shape, or
 // no room left in its rotary table, raises DEVERR_INDEX and the position is
 // clamped into range. (The same rule runs inside decide_norm_kernel when the
 // router is not forked onto a stream of its own.)
 __global__ void decode_decide_kernel(const float* scores, const float* thr, const int32_t* hdr, int B,
-                                     int C_max, int32_t* rows, int32_t* pos, int32_t* kept_out, int* err) {
+                                     int C_max, int32_t* lens, int32_t* rows, int32_t* pos, int32_t* kept_out,
+                                     int* err) {
   pdl_wait();
   pdl_trigger();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= B) return;
-  int t = hdr[0];
-  if (hdr[1] != C_max || t < 0 || t >= C_max) {
-    set_device_error(err, DEVERR_INDEX);
-    t = t < 0 ? 0 : (t >= C_max ? C_max - 1 : t);
-  }
-  const bool keep = scores[b] > thr[b];
-  rows[b] = keep ? b : -1;
-  pos[b] = t;
-  if (kept_out) kept_out[b] = keep ? 1 : 0;
+  if (b < B) decide_row(b, scores, thr, hdr, C_max, lens, rows, pos, kept_out, err);
 }
 
 // Attention of the new token of sequence b, query heads h G .. h G + G - 1
@@ -248,23 +242,37 @@ struct DecTc {
   static constexpr int RING = kDecStages * STAGE;
   static constexpr int OLD = HD + 8;                      // merge row stride (floats), padded
   static constexpr int MERGE = kDecWarps * 16 * (OLD + 2) * 4;
-  static_assert(MERGE <= RING, "the merge area reuses the ring");
-  static constexpr int SMEM = RING + 1024;                // + alignment slack
+  static constexpr int PART = 16 * (HD + 2) * 4;          // the split's result: [16][HD] and (max, sum) per head
+  static_assert(MERGE + PART <= RING, "the merge area reuses the ring");
+  static constexpr int QLD = HD + 8;                      // bf16 of a staged query row
+  static constexpr int SMEM = RING + 16 * QLD * 2 + 1024;   // + alignment slack
 };
 
-template <int HD>
+// The launch rotates the group's queries itself and, where its split holds the new
+// token's place, rotates and appends the token's key and value first (a proxy fence
+// and a barrier order them before the copy of that tile). With CLUSTER the splits
+// of a (sequence, head) are one cluster that combines its partials through
+// distributed shared memory. As a rotary + append launch, this one and a combine
+// launch the three took 19.1 us per layer at the Qwen2.5-7B shape (16 sequences, 750
+// cached tokens) and 12.9 us at the Pythia-160M shape (one sequence); one launch takes
+// 13.1 and 7.0 us. The arithmetic and its order are the same.
+
+template <int HD, bool CLUSTER>
 __global__ void __launch_bounds__(kDecTcThreads)
     decode_attn_tc_kernel(const __grid_constant__ CUtensorMap tk, const __grid_constant__ CUtensorMap tv,
-                          const bf16* qkv, int64_t ld, int Hq, int Hkv, const int32_t* lens, int C_max,
-                          int nsplit, float scale_log2, float* part_o, float2* part_ml, int* err,
-                          unsigned long long timeout_ns) {
+                          const bf16* qkv, int64_t ld, int Hq, int Hkv, const int32_t* lens, const int32_t* pos,
+                          const float2* tab, int half, bf16* kc, bf16* vc, int C_max,
+                          int nsplit, float scale_log2, float* part_o, float2* part_ml, bf16* out, int64_t ld_out,
+                          int* err, unsigned long long timeout_ns) {
   using C = DecTc<HD>;
   extern __shared__ __align__(1024) uint8_t dsm[];
-  __shared__ __align__(8) uint64_t bars[2 * kDecStages];
+  __shared__ __align__(8) uint64_t bars[2 * kDecStages + 1];
   __shared__ int abort_s;
   const uint32_t ring = (smem_u32(dsm) + 1023u) & ~1023u;
   uint8_t* ring_p = dsm + (ring - smem_u32(dsm));
+  bf16* sQ = reinterpret_cast<bf16*>(ring_p + C::RING);   // [16][QLD]
   const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[kDecStages]);
+  const uint32_t appended = smem_u32(&bars[2 * kDecStages]);
   volatile int* abort_flag = &abort_s;
   const int s = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
   const int G = Hq / Hkv;
@@ -274,6 +282,7 @@ __global__ void __launch_bounds__(kDecTcThreads)
       mbar_init(full0 + 8 * i, 1);
       mbar_init(empty0 + 8 * i, kDecWarps);
     }
+    mbar_init(appended, kDecWarps);
     abort_s = 0;
     fence_barrier_init();
   }
@@ -290,6 +299,10 @@ __global__ void __launch_bounds__(kDecTcThreads)
   dec_split_range(n, nsplit, s, lo, hi);
   const int ntiles = (hi - lo + kDecTK - 1) / kDecTK;
   const int row0 = (b * Hkv + h) * C_max + lo;            // first key's row in the layer's cache
+  const int pb = pos[b];
+  const float2* tab_row = tab + (int64_t)(pb & (kDecAppend - 1)) * half;
+  // this split holds the new token's place: its last tile waits for the append
+  const bool owner = (pb & kDecAppend) != 0 && n - 1 >= lo && n - 1 < hi;
 
   const int gid = lane >> 2, tig = lane & 3;
   float o[HD / 8][4];
@@ -304,6 +317,7 @@ __global__ void __launch_bounds__(kDecTcThreads)
       for (; t < ntiles; ++t) {
         const int st = t % kDecStages;
         if (!mbar_wait_bounded(empty0 + 8 * st, ((t / kDecStages) & 1) ^ 1, abort_flag, err, timeout_ns)) break;
+        if (owner && t == ntiles - 1 && !mbar_wait_bounded(appended, 0, abort_flag, err, timeout_ns)) break;
         const uint32_t fb = full0 + 8 * st;
         mbar_arrive_expect_tx(fb, C::STAGE);
         const uint32_t dk = ring + st * C::STAGE;
@@ -321,17 +335,60 @@ __global__ void __launch_bounds__(kDecTcThreads)
     }
   } else {
     // ------------------------------------------------------------ consumers
-    // Q of the group as A fragments (rows g >= G zero), once
+    // pairs k of a head's features: (k, k + half) of the rotated ones, then neighbours
+    auto pair_at = [&](int k, int& e0, int& e1) {
+      e0 = k < half ? k : 2 * half + 2 * (k - half);
+      e1 = k < half ? k + half : e0 + 1;
+    };
+    auto rotated = [&](const bf16* src, int k, int e0, int e1, bf16& ra, bf16& rc) {
+      ra = src[e0];
+      rc = src[e1];
+      if (k < half) {
+        const float2 cs = tab_row[k];
+        const float a = Elem<bf16>::to_f(ra), c = Elem<bf16>::to_f(rc);
+        ra = Elem<bf16>::from_f(a * cs.x - c * cs.y);
+        rc = Elem<bf16>::from_f(c * cs.x + a * cs.y);
+      }
+    };
+    const bf16* row = qkv + (int64_t)b * ld;
+    if (owner) {
+      // the new key (rotated) and value into the cache
+      const bf16* kn = row + (int64_t)(Hq + h) * HD;
+      const bf16* vn = kn + (int64_t)Hkv * HD;
+      const int64_t dst = (((int64_t)b * Hkv + h) * C_max + n - 1) * HD;
+      for (int k = threadIdx.x; k < HD / 2; k += 32 * kDecWarps) {
+        int e0, e1;
+        pair_at(k, e0, e1);
+        bf16 ra, rc;
+        rotated(kn, k, e0, e1, ra, rc);
+        kc[dst + e0] = ra;
+        kc[dst + e1] = rc;
+        *reinterpret_cast<uint32_t*>(vc + dst + 2 * k) = *reinterpret_cast<const uint32_t*>(vn + 2 * k);
+      }
+      asm volatile("fence.proxy.async;" ::: "memory");   // written by threads, read by the copies of the last tile
+      __syncwarp();
+      if (lane == 0) mbar_arrive(appended);
+    }
+    // the group's queries, rotated, as A fragments (rows g >= G zero), once
+    for (int i = threadIdx.x; i < 16 * (HD / 2); i += 32 * kDecWarps) {
+      const int g = i / (HD / 2), k = i % (HD / 2);
+      int e0, e1;
+      pair_at(k, e0, e1);
+      bf16 ra = __ushort_as_bfloat16(0), rc = ra;
+      if (g < G) rotated(row + (int64_t)(h * G + g) * HD, k, e0, e1, ra, rc);
+      sQ[g * C::QLD + e0] = ra;
+      sQ[g * C::QLD + e1] = rc;
+    }
+    named_bar_sync(1, 32 * kDecWarps);
     uint32_t qa[HD / 16][4];
-    const bf16* qrow = qkv + (int64_t)b * ld + (int64_t)h * G * HD;
-    const bool r0 = gid < G, r1 = gid + 8 < G;
 #pragma unroll
     for (int ks = 0; ks < HD / 16; ++ks) {
-      const int c = ks * 16 + tig * 2;
-      qa[ks][0] = r0 ? *reinterpret_cast<const uint32_t*>(qrow + gid * HD + c) : 0u;
-      qa[ks][1] = r1 ? *reinterpret_cast<const uint32_t*>(qrow + (gid + 8) * HD + c) : 0u;
-      qa[ks][2] = r0 ? *reinterpret_cast<const uint32_t*>(qrow + gid * HD + c + 8) : 0u;
-      qa[ks][3] = r1 ? *reinterpret_cast<const uint32_t*>(qrow + (gid + 8) * HD + c + 8) : 0u;
+      const bf16* q0 = sQ + gid * C::QLD + ks * 16 + tig * 2;
+      const bf16* q1 = q0 + 8 * C::QLD;
+      qa[ks][0] = *reinterpret_cast<const uint32_t*>(q0);
+      qa[ks][1] = *reinterpret_cast<const uint32_t*>(q1);
+      qa[ks][2] = *reinterpret_cast<const uint32_t*>(q0 + 8);
+      qa[ks][3] = *reinterpret_cast<const uint32_t*>(q1 + 8);
     }
     const int mi = lane >> 3, mr = lane & 7;   // ldmatrix: this lane's matrix and row
     for (int t = 0; t < ntiles; ++t) {
@@ -407,6 +464,8 @@ __global__ void __launch_bounds__(kDecTcThreads)
   __syncthreads();   // the ring is drained and read: its memory takes the merge
   float* mo = reinterpret_cast<float*>(ring_p);                     // [warp][16][OLD]
   float* mml = mo + kDecWarps * 16 * C::OLD;                        // [warp][16][2]
+  float* po = reinterpret_cast<float*>(ring_p + C::MERGE);          // [16][HD]
+  float2* pml = reinterpret_cast<float2*>(po + 16 * HD);            // [16]
   if (warp < kDecWarps) {
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
@@ -437,9 +496,36 @@ __global__ void __launch_bounds__(kDecTcThreads)
         ov += mo[(w * 16 + g) * C::OLD + e] * c;
       }
     }
-    const int64_t slot = ((int64_t)b * Hq + h * G + g) * nsplit + s;
-    part_o[slot * HD + e] = ov;
-    if (e == 0) part_ml[slot] = make_float2(m, l);
+    if (CLUSTER) {
+      po[g * HD + e] = ov;
+      if (e == 0) pml[g] = make_float2(m, l);
+    } else {
+      const int64_t slot = ((int64_t)b * Hq + h * G + g) * nsplit + s;
+      part_o[slot * HD + e] = ov;
+      if (e == 0) part_ml[slot] = make_float2(m, l);
+    }
+  }
+  if (CLUSTER) {
+    // every split's partial is in its CTA's shared memory: combined in split order, as
+    // decode_combine_kernel does, each CTA a share of the outputs
+    cluster_sync();
+    const uint32_t po_a = smem_u32(po), pml_a = smem_u32(pml);
+    for (int k = s * kDecTcThreads + threadIdx.x; k < G * HD; k += nsplit * kDecTcThreads) {
+      const int g = k / HD, e = k % HD;
+      float m = -INFINITY;
+      for (int q = 0; q < nsplit; ++q) m = fmaxf(m, ld_cluster_f32(map_to_cta(pml_a + 8 * g, q)));
+      float l = 0.f, o_sum = 0.f;
+      for (int q = 0; q < nsplit; ++q) {
+        const uint32_t pq = map_to_cta(pml_a + 8 * g, q);
+        const float mq = ld_cluster_f32(pq);
+        if (mq == -INFINITY) continue;
+        const float c = exp2f(mq - m);
+        l += ld_cluster_f32(pq + 4) * c;
+        o_sum += ld_cluster_f32(map_to_cta(po_a + 4 * k, q)) * c;
+      }
+      out[(int64_t)b * ld_out + (h * G + g) * HD + e] = Elem<bf16>::from_f(l > 0.f ? o_sum / l : 0.f);
+    }
+    cluster_sync();   // the partials stay until every CTA has read them
   }
 }
 
@@ -467,40 +553,34 @@ __global__ void decode_combine_kernel(const float* part_o, const float2* part_ml
   }
 }
 
-// Rotary embedding of the new tokens' query and key heads at their positions
-// (feature i < half pairs with i + half, as in the prefill), fused with the
-// cache append: a kept token's rotated key and its value join the layer's
-// cache at lens[b], then lens[b] += 1. One block per sequence b, wide enough
-// that each thread has one or two pairs (the launch is latency bound).
-template <typename T>
-__global__ void __launch_bounds__(kRopeThreads) rope_append_kernel(T* qkv, int64_t ld, int Hq, int Hkv, int hd, int half,
-                                   const int32_t* pos, const float2* tab, const int32_t* rows,
-                                   int32_t* lens, int C_max, T* kc, T* vc, int* err) {
+// fp32 storage: rotary embedding of the new tokens' query and key heads at their
+// positions (feature i < half pairs with i + half, as in the prefill), fused with the
+// cache append: a kept token's rotated key and its value join the layer's cache at
+// its counted place. One block per sequence b, wide enough that each thread has
+// one or two pairs (the launch is latency bound).
+__global__ void __launch_bounds__(kRopeThreads)
+    rope_append_kernel(float* qkv, int64_t ld, int Hq, int Hkv, int hd, int half, const int32_t* pos, const float2* tab,
+                       const int32_t* lens, int C_max, float* kc, float* vc) {
   pdl_wait();
   pdl_trigger();
   const int b = blockIdx.x;
-  T* row = qkv + (int64_t)b * ld;
+  float* row = qkv + (int64_t)b * ld;
   const int q = Hq * hd, kvw = Hkv * hd;
-  bool append = rows[b] >= 0;
-  const int len = lens[b];
-  if (append && (len < 0 || len >= C_max)) {
-    if (threadIdx.x == 0) set_device_error(err, DEVERR_INDEX);
-    append = false;
-  }
-  const float2* tab_row = tab + (int64_t)pos[b] * half;
+  const int pb = pos[b];
+  const bool append = (pb & kDecAppend) != 0;
+  const int place = lens[b] - 1;
+  const float2* tab_row = tab + (int64_t)(pb & (kDecAppend - 1)) * half;
   // rotated pairs of every query and key head
   for (int k = threadIdx.x; k < (Hq + Hkv) * half; k += blockDim.x) {
     const int h = k / half, i = k % half;
-    T* base = row + (int64_t)h * hd;
+    float* base = row + (int64_t)h * hd;
     const float2 cs = tab_row[i];
-    const float a = Elem<T>::to_f(base[i]);
-    const float c = Elem<T>::to_f(base[i + half]);
-    const T ra = Elem<T>::from_f(a * cs.x - c * cs.y);
-    const T rc = Elem<T>::from_f(c * cs.x + a * cs.y);
+    const float a = base[i], c = base[i + half];
+    const float ra = a * cs.x - c * cs.y, rc = c * cs.x + a * cs.y;
     base[i] = ra;
     base[i + half] = rc;
     if (append && h >= Hq) {
-      const int64_t dst = (((int64_t)b * Hkv + (h - Hq)) * C_max + len) * hd;
+      const int64_t dst = (((int64_t)b * Hkv + (h - Hq)) * C_max + place) * hd;
       kc[dst + i] = ra;
       kc[dst + i + half] = rc;
     }
@@ -509,13 +589,11 @@ __global__ void __launch_bounds__(kRopeThreads) rope_append_kernel(T* qkv, int64
     // key features past the rotary pairs, and the values
     for (int c = threadIdx.x; c < kvw; c += blockDim.x) {
       const int h = c / hd, e = c % hd;
-      const int64_t dst = (((int64_t)b * Hkv + h) * C_max + len) * hd + e;
+      const int64_t dst = (((int64_t)b * Hkv + h) * C_max + place) * hd + e;
       if (e >= 2 * half) kc[dst] = row[q + c];
       vc[dst] = row[q + kvw + c];
     }
   }
-  __syncthreads();
-  if (threadIdx.x == 0 && append) lens[b] = len + 1;
 }
 
 __global__ void decode_advance_kernel(int32_t* hdr) {
@@ -559,31 +637,31 @@ cudaError_t cache_header(int32_t* hdr, int T, int C_max, int L, int B, const Dev
   return launch_pdl(cache_header_kernel, dim3(1), dim3(32), 0, dev.stream, hdr, T, C_max, L, B);
 }
 
-template <int HD>
-static cudaError_t launch_decode_tc(const CUtensorMap& tk, const CUtensorMap& tv, const bf16* qkv, int64_t ld,
-                                    int Hq, int Hkv, const int32_t* lens, int C_max, int B, int ns,
-                                    float scale_log2, float* part_o, float2* part_ml, const Dev& dev) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(decode_attn_tc_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         DecTc<HD>::SMEM);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
-  return launch_pdl(decode_attn_tc_kernel<HD>, dim3(ns, Hkv, B), dim3(kDecTcThreads), (size_t)DecTc<HD>::SMEM,
-                    dev.stream, tk, tv, qkv, ld, Hq, Hkv, lens, C_max, ns, scale_log2, part_o, part_ml, dev.err,
-                    kWaitTimeoutNs);
+template <int HD, bool CLUSTER>
+static cudaError_t launch_decode_tc(const CUtensorMap& tk, const CUtensorMap& tv, const DecodeAttn& a, int ns,
+                                    float scale_log2, const Dev& dev) {
+  const cudaError_t e = allow_smem(decode_attn_tc_kernel<HD, CLUSTER>, DecTc<HD>::SMEM);
+  if (e != cudaSuccess) return e;
+  const dim3 grid(ns, a.Hkv, a.B);
+  const bf16* q = static_cast<const bf16*>(a.qkv);
+  bf16 *kc = static_cast<bf16*>(a.kc), *vc = static_cast<bf16*>(a.vc), *out = static_cast<bf16*>(a.out);
+  if (CLUSTER)
+    return launch_pdl_cluster(decode_attn_tc_kernel<HD, CLUSTER>, grid, dim3(kDecTcThreads), (size_t)DecTc<HD>::SMEM,
+                              dev.stream, ns, tk, tv, q, a.ld, a.Hq, a.Hkv, a.lens, a.pos, a.tab, a.half, kc, vc,
+                              a.C_max, ns, scale_log2, a.part_o, a.part_ml, out, a.ld_out, dev.err, kWaitTimeoutNs);
+  return launch_pdl(decode_attn_tc_kernel<HD, CLUSTER>, grid, dim3(kDecTcThreads), (size_t)DecTc<HD>::SMEM, dev.stream,
+                    tk, tv, q, a.ld, a.Hq, a.Hkv, a.lens, a.pos, a.tab, a.half, kc, vc, a.C_max, ns, scale_log2,
+                    a.part_o, a.part_ml, out, a.ld_out, dev.err, kWaitTimeoutNs);
 }
 
-cudaError_t decode_decide(const float* scores, const float* thr, const int32_t* hdr, int B, int C_max,
+cudaError_t decode_decide(const float* scores, const float* thr, const int32_t* hdr, int B, int C_max, int32_t* lens,
                           int32_t* rows, int32_t* pos, int32_t* kept_out, const Dev& dev) {
   return launch_pdl(decode_decide_kernel, dim3((B + 127) / 128), dim3(128), 0, dev.stream, scores, thr, hdr, B,
-                    C_max, rows, pos, kept_out, dev.err);
+                    C_max, lens, rows, pos, kept_out, dev.err);
 }
 
-cudaError_t decode_attention(int dtype, const void* qkv, int64_t ld, int Hq, int Hkv, int hd, const void* kc,
-                             const void* vc, const int32_t* lens, int C_max, int B, float* part_o,
-                             float2* part_ml, void* out, int64_t ld_out, const Dev& dev) {
+cudaError_t decode_attention(int dtype, const DecodeAttn& a, const Dev& dev) {
+  const int B = a.B, Hq = a.Hq, Hkv = a.Hkv, hd = a.hd, C_max = a.C_max;
   if (B <= 0) return cudaSuccess;
   if (Hq % Hkv != 0 || Hq / Hkv > kMaxGroup || (hd != 64 && hd != 128)) return cudaErrorInvalidValue;
   const int ns = decode_splits(B, Hkv, C_max, dev.num_sms);
@@ -596,37 +674,28 @@ cudaError_t decode_attention(int dtype, const void* qkv, int64_t ld, int Hq, int
     const int64_t rows = (int64_t)B * Hkv * C_max;
     if (rows + kDecTK > INT32_MAX) return cudaErrorInvalidValue;
     CUtensorMap tk, tv;
-    if (!make_tmap_bf16(&tk, kc, (uint64_t)rows, (uint64_t)hd, (uint64_t)hd, 64, kDecTK) ||
-        !make_tmap_bf16(&tv, vc, (uint64_t)rows, (uint64_t)hd, (uint64_t)hd, 64, kDecTK))
+    if (!make_tmap_bf16(&tk, a.kc, (uint64_t)rows, (uint64_t)hd, (uint64_t)hd, 64, kDecTK) ||
+        !make_tmap_bf16(&tv, a.vc, (uint64_t)rows, (uint64_t)hd, (uint64_t)hd, 64, kDecTK))
       return cudaErrorInvalidValue;
-    const bf16* q = static_cast<const bf16*>(qkv);
-    e = hd == 128 ? launch_decode_tc<128>(tk, tv, q, ld, Hq, Hkv, lens, C_max, B, ns, scale_log2, part_o, part_ml, dev)
-                  : launch_decode_tc<64>(tk, tv, q, ld, Hq, Hkv, lens, C_max, B, ns, scale_log2, part_o, part_ml, dev);
-  } else {
-    e = launch_pdl(decode_attn_f32_kernel, dim3(ns, Hkv, B), dim3(kDecThreads), 0, dev.stream,
-                   static_cast<const float*>(qkv), ld, Hq, Hkv, hd, static_cast<const float*>(kc),
-                   static_cast<const float*>(vc), lens, C_max, ns, scale_log2, part_o, part_ml);
+    // up to 8 splits (a portable cluster) combine inside the launch, more need a launch of their own
+    if (ns <= 8)
+      return hd == 128 ? launch_decode_tc<128, true>(tk, tv, a, ns, scale_log2, dev)
+                       : launch_decode_tc<64, true>(tk, tv, a, ns, scale_log2, dev);
+    e = hd == 128 ? launch_decode_tc<128, false>(tk, tv, a, ns, scale_log2, dev)
+                  : launch_decode_tc<64, false>(tk, tv, a, ns, scale_log2, dev);
+    if (e != cudaSuccess) return e;
+    return launch_pdl(decode_combine_kernel<bf16>, dim3(Hq, B), dim3(128), 0, dev.stream, a.part_o, a.part_ml, Hq,
+                      hd, ns, static_cast<bf16*>(a.out), a.ld_out);
   }
+  e = launch_pdl(rope_append_kernel, dim3(B), dim3(kRopeThreads), 0, dev.stream, static_cast<float*>(a.qkv), a.ld, Hq, Hkv,
+                 hd, a.half, a.pos, a.tab, a.lens, C_max, static_cast<float*>(a.kc), static_cast<float*>(a.vc));
   if (e != cudaSuccess) return e;
-  if (dtype == kBF16)
-    return launch_pdl(decode_combine_kernel<bf16>, dim3(Hq, B), dim3(128), 0, dev.stream, part_o, part_ml, Hq,
-                      hd, ns, static_cast<bf16*>(out), ld_out);
-  return launch_pdl(decode_combine_kernel<float>, dim3(Hq, B), dim3(128), 0, dev.stream, part_o, part_ml, Hq, hd,
-                    ns, static_cast<float*>(out), ld_out);
-}
-
-cudaError_t rope_append(int dtype, void* qkv, int64_t ld, int Hq, int Hkv, int hd, int rotary_dim, int B,
-                        const int32_t* rows, const int32_t* pos, const float2* tab, int32_t* lens, int C_max,
-                        void* kc, void* vc, const Dev& dev) {
-  if (B <= 0) return cudaSuccess;
-  const int half = rotary_dim / 2;
-  if (dtype == kBF16)
-    return launch_pdl(rope_append_kernel<bf16>, dim3(B), dim3(kRopeThreads), 0, dev.stream, static_cast<bf16*>(qkv), ld, Hq,
-                      Hkv, hd, half, pos, tab, rows, lens, C_max, static_cast<bf16*>(kc), static_cast<bf16*>(vc),
-                      dev.err);
-  return launch_pdl(rope_append_kernel<float>, dim3(B), dim3(kRopeThreads), 0, dev.stream, static_cast<float*>(qkv), ld, Hq,
-                    Hkv, hd, half, pos, tab, rows, lens, C_max, static_cast<float*>(kc), static_cast<float*>(vc),
-                    dev.err);
+  e = launch_pdl(decode_attn_f32_kernel, dim3(ns, Hkv, B), dim3(kDecThreads), 0, dev.stream,
+                 static_cast<const float*>(a.qkv), a.ld, Hq, Hkv, hd, static_cast<const float*>(a.kc),
+                 static_cast<const float*>(a.vc), a.lens, C_max, ns, scale_log2, a.part_o, a.part_ml);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(decode_combine_kernel<float>, dim3(Hq, B), dim3(128), 0, dev.stream, a.part_o, a.part_ml, Hq, hd,
+                    ns, static_cast<float*>(a.out), a.ld_out);
 }
 
 cudaError_t decode_advance(int32_t* hdr, const Dev& dev) {

@@ -213,22 +213,30 @@ cudaError_t kv_fill(int dtype, const void* qkv, int64_t ld, int q, int kvw, int 
 cudaError_t kv_threshold(const float* scores, const int32_t* idx, int B, int T, int K, int32_t* lens,
                          float* thr, const Dev& dev);
 cudaError_t cache_header(int32_t* hdr, int T, int C_max, int L, int B, const Dev& dev);
-// Keep decision of each new token (one per sequence) at one layer (decode.cu).
-cudaError_t decode_decide(const float* scores, const float* thr, const int32_t* hdr, int B, int C_max,
+// Keep decision of each new token (one per sequence) at one layer, its count in
+// the layer's cache included (decode.cu).
+cudaError_t decode_decide(const float* scores, const float* thr, const int32_t* hdr, int B, int C_max, int32_t* lens,
                           int32_t* rows, int32_t* pos, int32_t* kept_out, const Dev& dev);
-// Keep decision of each new token (one per sequence) at one layer, fused with
-// the norm(s) of the B new rows (rowwise.cu).
+// The same, fused with the norm(s) of the B new rows (rowwise.cu).
 cudaError_t decide_norm(int dtype, const void* x, int B, int d, bool is_rms, const void* g1, const void* b1,
                         const void* g2, const void* b2, float eps, void* out1, void* out2, const float* scores,
-                        const float* thr, const int32_t* hdr, int C_max, int32_t* rows, int32_t* pos,
+                        const float* thr, const int32_t* hdr, int C_max, int32_t* lens, int32_t* rows, int32_t* pos,
                         int32_t* kept_out, const Dev& dev);
-cudaError_t decode_attention(int dtype, const void* qkv, int64_t ld, int Hq, int Hkv, int hd, const void* kc,
-                             const void* vc, const int32_t* lens, int C_max, int B, float* part_o,
-                             float2* part_ml, void* out, int64_t ld_out, const Dev& dev);
-// Rotary embedding of the decode rows fused with the cache append (rotary_dim 0: append only).
-cudaError_t rope_append(int dtype, void* qkv, int64_t ld, int Hq, int Hkv, int hd, int rotary_dim, int B,
-                        const int32_t* rows, const int32_t* pos, const float2* tab, int32_t* lens, int C_max,
-                        void* kc, void* vc, const Dev& dev);
+// Set in pos[b] beside the position: the new token is counted in the layer's cache
+// and its key and value are to be appended.
+constexpr int kDecAppend = 1 << 30;
+// Attention of the new tokens over the layer's cache, their rotary and the cache
+// append included.
+struct DecodeAttn {
+  void* qkv; int64_t ld;             // [B][q + 2 kv], not yet rotated (fp32: rotated in place)
+  int Hq, Hkv, hd, half, C_max, B;   // half: rotary pairs
+  void *kc, *vc;                     // the layer's cache
+  const int32_t *lens, *pos;         // counts (the new tokens included), positions with kDecAppend
+  const float2* tab;                 // [C_max][half]
+  float* part_o; float2* part_ml;    // split partials
+  void* out; int64_t ld_out;
+};
+cudaError_t decode_attention(int dtype, const DecodeAttn& a, const Dev& dev);
 cudaError_t decode_advance(int32_t* hdr, const Dev& dev);
 
 }  // namespace adadsf

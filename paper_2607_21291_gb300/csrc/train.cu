@@ -341,19 +341,6 @@ __global__ void __launch_bounds__(kRrThreads, 2)
   if (j0 == 0) ds_out[m] = ds;
 }
 
-// Router gradient, part 2: dW1[j][k] = sum_m du[m][j] x[rows[m]][k]. A cluster
-// of 8 CTAs owns 64 columns k and all h <= 64 units; each CTA sums an eighth
-// of the rows (rows staged 32 at a time with the next 32 in flight) and the
-// eighths are added in rank order through distributed shared memory. The split
-// along m is what fills the GPU: the output has only d / 64 such tiles (32 at d =
-// 2048). fp32 x: 8 units x 4 columns a thread on FFMA. bf16 x: tensor products with
-// du cut into three bf16 parts that add up to it exactly (8 of its 24 bits each), the
-// smallest first, each 16 rows summed from zero and added in fp32, so nothing of
-// du's precision is lost. The last cluster sums db1[j] = sum_m du[m][j], dw2[j] = sum_m
-// ds[m] SiLU(u)[m][j] and db2 = sum_m ds[m] the same way. With part 1 it takes
-// 29 us at M = 2048, d = 2048 (bf16) and 0.42 ms at M = 32768; 76 us and 0.97
-// ms with both parts on FFMA, 1024 us and 20.8 ms for one warp a row with 64 serial
-// dots and a reduction of 17 blocks that summed the vectors in one thread each.
 __device__ __forceinline__ void ldsm_x4_trans(uint32_t addr, uint32_t (&r)[4]) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
@@ -370,6 +357,19 @@ __device__ __forceinline__ void bf16_parts(float f, uint32_t (&p)[3]) {
   p[2] = finite ? __float_as_uint(r - __uint_as_float(p[1])) & 0xffff0000u : 0u;
 }
 
+// Router gradient, part 2: dW1[j][k] = sum_m du[m][j] x[rows[m]][k]. A cluster
+// of 8 CTAs owns 64 columns k and all h <= 64 units; each CTA sums an eighth
+// of the rows (rows staged 32 at a time with the next 32 in flight) and the
+// eighths are added in rank order through distributed shared memory. The split
+// along m is what fills the GPU: the output has only d / 64 such tiles (32 at d =
+// 2048). fp32 x: 8 units x 4 columns a thread on FFMA. bf16 x: tensor products with
+// du cut into three bf16 parts that add up to it exactly (8 of its 24 bits each), the
+// smallest first, each 16 rows summed from zero and added in fp32, so nothing of
+// du's precision is lost. The last cluster sums db1[j] = sum_m du[m][j], dw2[j] = sum_m
+// ds[m] SiLU(u)[m][j] and db2 = sum_m ds[m] the same way. With part 1 it takes
+// 29 us at M = 2048, d = 2048 (bf16) and 0.42 ms at M = 32768; 76 us and 0.97
+// ms with both parts on FFMA, 1024 us and 20.8 ms for one warp a row with 64 serial
+// dots and a reduction of 17 blocks that summed the vectors in one thread each.
 constexpr int kRedCluster = 8;
 constexpr int kRedThreads = 128;
 constexpr int kRedCols = 64;
