@@ -13,7 +13,7 @@
  *  - Device pointers must be 16-byte aligned; the workspace 256-byte aligned.
  *  - `stream` is a cudaStream_t passed as void* (NULL = legacy default
  *    stream). Every device entry point only enqueues work on that stream
- *    (adadsf_decode_step also on a stream of its own that it joins back into
+ *    (adadsf_decode_step may use a stream of its own that it joins back into
  *    it) and returns without synchronising; results are ready once the
  *    stream is.
  *  - Tensors are dense row-major. Weights are [out_features, in_features]
@@ -433,14 +433,14 @@ adadsf_status adadsf_sparse_model_forward(const adadsf_model_cfg *cfg, const ada
  * the workspace of adadsf_model_workspace_size(cfg, B, T, K_host, 0); a
  * decode step adadsf_decode_workspace_size(cfg, B, C_max), and at most 16
  * query heads per key/value head (else ADADSF_ERR_UNSUPPORTED).
- * A decode step runs each layer's router and keep decision on a second
- * stream owned by the library, beside the norm and QKV projection on
- * `stream`. Events fork that stream from `stream` and join it back before
- * the layer's cache append, so the step is complete when `stream` is, and a
- * graph captured from `stream` contains it. The second stream is made on
- * the first decode step enqueued on `stream`; a step captured before any
- * uncaptured step on that stream runs on `stream` alone, with the same
- * results.
+ * A bf16 step of at most 16 sequences runs on `stream` alone. Any other step
+ * runs each layer's router and keep decision on a second stream owned by the
+ * library, beside the norm and QKV projection on `stream`. Events fork that
+ * stream from `stream` and join it back before the layer's cache append, so
+ * the step is complete when `stream` is, and a graph captured from `stream`
+ * contains it. The second stream is made on the first such step enqueued on
+ * `stream`; a step captured before any uncaptured one on that stream runs on
+ * `stream` alone, with the same results.
  * ---------------------------------------------------------------------- */
 size_t adadsf_kv_cache_size(const adadsf_model_cfg *cfg, int B, int C_max);
 adadsf_status adadsf_prefill(const adadsf_model_cfg *cfg, const adadsf_model_weights *w,
@@ -486,7 +486,7 @@ typedef enum {
   ADADSF_KERNEL_GEMM_QKV_UP,   /* GPT-NeoX: QKV and MLP-up projections in one launch */
   ADADSF_KERNEL_GEMM_O_DOWN,   /* GPT-NeoX: output + MLP-down projections, one accumulator */
   ADADSF_KERNEL_TOPK_GATHER_NORM, /* Top-K fused with the gather and norms of the kept rows */
-  ADADSF_KERNEL_DECIDE,        /* decode: keep decision of each new token (inside the norm launch when the step runs on one stream) */
+  ADADSF_KERNEL_DECIDE,        /* decode: keep decision of each new token (with the router and norm for at most 16 bf16 sequences; inside the norm launch when another step runs on one stream) */
   ADADSF_KERNEL_KV_CACHE,      /* decode cache: fill (prefill), thresholds */
   ADADSF_KERNEL_ALIGN,         /* alignment objective and router gradient (Eqs. 9-10) */
   ADADSF_KERNEL_COUNT

@@ -380,6 +380,8 @@ adadsf_status layer_impl(const adadsf_model_cfg* c, const adadsf_layer_weights* 
   // decode on two streams: the router and the keep decision on the side
   // stream (from the layer input x), the norm and QKV on the main one
   const bool forked = dec && dec->side;
+  // few sequences: router, decision and norm in one launch instead
+  const bool front = dec && decode_front_fits(dt, B, c->router_hidden);
   Dev sdev = dev;
   if (forked) {
     sdev.stream = dec->side;
@@ -391,7 +393,7 @@ adadsf_status layer_impl(const adadsf_model_cfg* c, const adadsf_layer_weights* 
   // squares, the projection loads the kept rows of x by row gathers, and its
   // epilogue scales each row by 1 / rms before the bias and rotary.
   const bool fuse1 = tc && !dec && !dense && !neox && gathered_qkv(c) && lb.tsq && M > 32LL * dev.num_sms;
-  if (!dense || gate || sink) {
+  if ((!dense || gate || sink) && !front) {
     const double rf = 2.0 * BT * c->router_hidden * d;
     const double rb = (double)BT * d * es + (double)c->router_hidden * d * es + BT * 4.0;
     // a2: router scores of every token (bf16: tensor cores, tiles split
@@ -411,7 +413,25 @@ adadsf_status layer_impl(const adadsf_model_cfg* c, const adadsf_layer_weights* 
     // decode: keep decision of each new token and the norms of all B rows
     // (a bypassing token's block output is computed and dropped: the
     // projections stream their weights once either way)
-    if (forked) {
+    if (front) {
+      DecodeFront f;
+      f.x = x;
+      f.B = B;
+      f.d = d;
+      f.w1 = w->router_w1; f.rb1 = w->router_b1; f.w2 = w->router_w2; f.rb2 = w->router_b2;
+      f.g1 = w->ln1_w; f.b1 = w->ln1_b; f.g2 = w->ln2_w; f.b2 = w->ln2_b;
+      f.eps = c->norm_eps;
+      f.out1 = lb.n1;
+      f.out2 = neox ? lb.n2 : nullptr;
+      f.scores = lb.scores;
+      f.thr = dec->thr;
+      f.hdr = dec->hdr;
+      f.C_max = dec->C_max;
+      f.lens = dec->lens; f.rows = dec->rows; f.pos = dec->pos; f.kept_out = dec->kept_out;
+      TRY(launch(dev, ADADSF_KERNEL_DECIDE, false, 2.0 * B * c->router_hidden * d,
+                 Md * es * (neox ? 3 : 2) + (double)c->router_hidden * d * es + 16.0 * B,
+                 CALL(decode_front(f, !neox, dev), "router + keep decision + norm")));
+    } else if (forked) {
       TRY(launch(sdev, ADADSF_KERNEL_DECIDE, false, 0, 16.0 * B,
                  CALL(decode_decide(lb.scores, dec->thr, dec->hdr, B, dec->C_max, dec->lens, dec->rows, dec->pos,
                                     dec->kept_out, sdev),
@@ -1511,7 +1531,8 @@ adadsf_status adadsf_decode_step(const adadsf_model_cfg* cfg, const adadsf_model
   lb.tsq = ds.layer.tsq ? at<float>(ws, ds.layer.tsq) : nullptr;
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-  const bool has_side = decode_side_stream(dev.stream, &side, &ev_fork, &ev_join);
+  const bool has_side = !decode_front_fits(dt, B, cfg->router_hidden) &&
+                        decode_side_stream(dev.stream, &side, &ev_fork, &ev_join);
   for (int l = 0; l < cfg->n_layers; ++l) {
     DecodeCtx dc;
     dc.thr = cv.thr + (int64_t)l * B;

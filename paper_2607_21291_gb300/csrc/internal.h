@@ -222,6 +222,22 @@ cudaError_t decide_norm(int dtype, const void* x, int B, int d, bool is_rms, con
                         const void* g2, const void* b2, float eps, void* out1, void* out2, const float* scores,
                         const float* thr, const int32_t* hdr, int C_max, int32_t* lens, int32_t* rows, int32_t* pos,
                         int32_t* kept_out, const Dev& dev);
+// Router score, keep decision and norm(s) of the new rows in one launch (rowwise.cu;
+// bf16, at most 16 sequences, 64 router units).
+struct DecodeFront {
+  const void* x;                              // [B][d]
+  int B, d;
+  const void *w1, *rb1, *w2, *rb2;            // router
+  const void *g1, *b1, *g2, *b2;              // norms (b1, g2, b2: GPT-NeoX)
+  float eps;
+  void *out1, *out2;                          // out2 or null
+  float* scores;
+  const float* thr; const int32_t* hdr;
+  int C_max;
+  int32_t *lens, *rows, *pos, *kept_out;
+};
+bool decode_front_fits(int dtype, int B, int h);
+cudaError_t decode_front(const DecodeFront& a, bool is_rms, const Dev& dev);
 // Set in pos[b] beside the position: the new token is counted in the layer's cache
 // and its key and value are to be appended.
 constexpr int kDecAppend = 1 << 30;

@@ -146,34 +146,42 @@ __device__ __forceinline__ void mma_16816(float (&d)[4], uint32_t a0, uint32_t a
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-__device__ __forceinline__ float4 router_rows_units_mma(const bf16* xr0, const bf16* xr1, const bf16* w1, int d,
-                                                        float* smem) {
+// One piece of 32 features of the operands, in flight.
+struct RouterPiece {
+  uint4 w[8], xa, xb;
+  __device__ __forceinline__ void load_w(const bf16* w1, int d, int c) {
+    const int lane = threadIdx.x & 31;
+    const int64_t k = (int64_t)c * 32 + (lane & 3) * 8;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = *reinterpret_cast<const uint4*>(w1 + (int64_t)(8 * i + (lane >> 2)) * d + k);
+  }
+  __device__ __forceinline__ void load_x(const bf16* xr0, const bf16* xr1, int c) {
+    const int64_t k = (int64_t)c * 32 + (threadIdx.x & 3) * 8;
+    xa = *reinterpret_cast<const uint4*>(xr0 + k);
+    xb = *reinterpret_cast<const uint4*>(xr1 + k);
+  }
+};
+// The sums over pieces [c_lo, c_hi), which the warps take in turn; `next` holds the
+// weights of the warp's first piece (c_lo + warp) if there is one.
+__device__ __forceinline__ float4 router_rows_partial(const bf16* xr0, const bf16* xr1, const bf16* w1, int d, int c_lo,
+                                                      int c_hi, RouterPiece& next, float* smem) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int gid = lane >> 2, tig = lane & 3;
   float tot[8][4];
 #pragma unroll
   for (int i = 0; i < 8; ++i) tot[i][0] = tot[i][1] = tot[i][2] = tot[i][3] = 0.f;
-  const int n = d / 32;
-  uint4 wv[8], xa, xb;
-  auto fetch = [&](int c) {
-    const int64_t k = (int64_t)c * 32 + tig * 8;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) wv[i] = *reinterpret_cast<const uint4*>(w1 + (int64_t)(8 * i + gid) * d + k);
-    xa = *reinterpret_cast<const uint4*>(xr0 + k);
-    xb = *reinterpret_cast<const uint4*>(xr1 + k);
-  };
-  if (warp < n) fetch(warp);
-  for (int c = warp; c < n; c += kRrWarps) {
-    uint4 w[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) w[i] = wv[i];
-    const uint4 a = xa, b = xb;
-    if (c + kRrWarps < n) fetch(c + kRrWarps);
+  if (c_lo + warp < c_hi) next.load_x(xr0, xr1, c_lo + warp);
+  for (int c = c_lo + warp; c < c_hi; c += kRrWarps) {
+    const RouterPiece cur = next;
+    if (c + kRrWarps < c_hi) {
+      next.load_w(w1, d, c + kRrWarps);
+      next.load_x(xr0, xr1, c + kRrWarps);
+    }
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       float p[4] = {0.f, 0.f, 0.f, 0.f};
-      mma_16816(p, a.x, b.x, a.y, b.y, w[i].x, w[i].y);
-      mma_16816(p, a.z, b.z, a.w, b.w, w[i].z, w[i].w);
+      mma_16816(p, cur.xa.x, cur.xb.x, cur.xa.y, cur.xb.y, cur.w[i].x, cur.w[i].y);
+      mma_16816(p, cur.xa.z, cur.xb.z, cur.xa.w, cur.xb.w, cur.w[i].z, cur.w[i].w);
 #pragma unroll
       for (int e = 0; e < 4; ++e) tot[i][e] += p[e];
     }

@@ -308,10 +308,13 @@ __global__ void __launch_bounds__(kRrThreads, 2)
   const int64_t mb = m0 + (lane >> 2) + 8 < M ? m0 + (lane >> 2) + 8 : M - 1;
   // its barriers make gd_s visible
   float4 u4;
-  if constexpr (sizeof(T) == 2)
-    u4 = router_rows_units_mma(x + (int64_t)rows[ma] * d, x + (int64_t)rows[mb] * d, w1, d, smem_rr);
-  else
+  if constexpr (sizeof(T) == 2) {
+    RouterPiece first;
+    if (warp < d / 32) first.load_w(w1, d, warp);
+    u4 = router_rows_partial(x + (int64_t)rows[ma] * d, x + (int64_t)rows[mb] * d, w1, d, 0, d / 32, first, smem_rr);
+  } else {
     u4 = router_rows_units<T>(x + (int64_t)rows[ma] * d, x + (int64_t)rows[mb] * d, w1, 0, h, d, smem_rr);
+  }
   const int row = threadIdx.x >> 4, j0 = (threadIdx.x & 15) * 4;
   const float uu[4] = {u4.x, u4.y, u4.z, u4.w};
   float si[4], dsi[4], s = 0.f;

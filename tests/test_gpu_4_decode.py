@@ -44,6 +44,14 @@ CASES = [
     (NEOX_F32, 2, 40, [20, 40], 4, 48, False, None),
     (QWEN7_ATTN, 2, 700, [350, 700], 3, 720, False, H.BF16_DEEP_ELEM_TOL),
     (QWEN_G16, 3, 200, [131, 64], 3, 216, True, None),
+    # 16 and 17 sequences: the last batch whose router, decision and norm are one
+    # launch, and the first that takes the second stream; 9 to fill a second
+    # half tile; a cache that needs more splits than a cluster combines (a 700-token
+    # prompt through two layers and the final norm: the deep bound, as above)
+    (QWEN_SMALL, 16, 40, [20, 40, 13], 3, 48, True, None),
+    (NEOX_SMALL, 17, 40, [20, 40, 13], 3, 48, False, None),
+    (NEOX_SMALL, 9, 33, [20, 33, 13], 3, 40, False, None),
+    (QWEN_G16, 2, 700, [500, 700], 3, 720, False, H.BF16_DEEP_ELEM_TOL),
 ]
 
 
