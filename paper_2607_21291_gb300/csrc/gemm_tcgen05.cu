@@ -1739,6 +1739,7 @@ size_t gemm_split_scratch_bytes() { return (size_t)160 * BM * 256 * 4; }
 cudaError_t gemm_bf16(const GemmArgs& a, const Dev& dev) {
   if (a.M <= 0) return cudaSuccess;
   if (a.a_gather && (a.epi.act == ACT_SWIGLU || a.a_gather_rows <= 0)) return cudaErrorInvalidValue;
+  if (gemm_rows_takes(a, nullptr)) return gemm_rows(a, nullptr, dev);
   // SwiGLU: 256 x 128 gate/up tiles on CTA pairs when that still gives every
   // pair of SMs at least two tiles.
   if (a.epi.act == ACT_SWIGLU) {
@@ -1759,6 +1760,7 @@ cudaError_t gemm_bf16_grouped(const GemmArgs& a, const GemmArgs& b, const Dev& d
     return g.epi.act != ACT_SWIGLU && g.K2 == 0;
   };
   if (!plain(a) || !plain(b)) return cudaErrorInvalidValue;
+  if (gemm_rows_takes(a, &b)) return gemm_rows(a, &b, dev);
   // Fewest rounds of tiles (a k-block costs the same for any tile width);
   // ties go to CTA pairs (half the weight bytes per SM), then to 256-wide
   // tiles. Problem `a` comes first in the tile order: pass the one with the

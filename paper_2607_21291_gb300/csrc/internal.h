@@ -125,6 +125,10 @@ cudaError_t gemm_bf16(const GemmArgs& a, const Dev& dev);
 // Two independent plain projections (no SwiGLU, router or second K source)
 // in one launch.
 cudaError_t gemm_bf16_grouped(const GemmArgs& a, const GemmArgs& b, const Dev& dev);
+// gemm_rows.cu -- bf16 projections of at most 16 rows and few weights (b: a second
+// problem on the same number of rows, or null).
+bool gemm_rows_takes(const GemmArgs& a, const GemmArgs* b);
+cudaError_t gemm_rows(const GemmArgs& a, const GemmArgs* b, const Dev& dev);
 // train.cu -- alignment objective (Eqs. 9-10) and the router gradient.
 int train_row_blocks(int64_t n);
 cudaError_t align_hidden(int dtype, const void* hs, const void* hd, int64_t n_rows, int d, float* grad,

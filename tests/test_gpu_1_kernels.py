@@ -146,6 +146,26 @@ def test_linear_f32(A, M, N, Kd):
     assert H.max_rel(H.to_np(out), O.linear(x, w, None, "gelu")) < 1e-5
 
 
+@pytest.mark.parametrize("M,N,Kd,act", [(1, 64, 64, 0), (7, 192, 448, 1), (8, 3072, 768, 1), (9, 2304, 768, 0),
+                                        (16, 64, 3072, 0), (16, 4096, 1984, 1), (8, 1536, 8960, 0), (17, 768, 768, 0)])
+def test_linear_bf16_few_rows(A, M, N, Kd, act):
+    """Products of at most 16 rows: one and two 8-row halves, fewer pieces of K
+    than warps and not a multiple of them, single and several tiles a block (and
+    17 rows, which take the tensor-core kernels). One bf16 rounding of the output
+    (2^-9 of an element, under 8e-3 of the largest)."""
+    g = np.random.default_rng(M * N + Kd)
+    x = S.round_to(g.standard_normal((M, Kd)).astype(np.float32), "bf16")
+    w = S.round_to((g.standard_normal((N, Kd)) / np.sqrt(Kd)).astype(np.float32), "bf16")
+    b = S.round_to(g.standard_normal(N).astype(np.float32), "bf16")
+    out = torch.full((M + 1, N), 7.0, dtype=torch.bfloat16, device="cuda")
+    ws = A.workspace(A.LINEAR_SPLIT_WS_BYTES)
+    A.adadsf_linear(*(H.to_dev(t, torch.bfloat16) for t in (x, w, b)), out[:M], act=act, ws=ws)
+    assert A.adadsf_sync_check(ws) == A.OK
+    ref = O.linear(x, w, b.astype(np.float64), "gelu" if act else None)
+    assert H.max_rel(H.to_np(out[:M]), ref) < 8e-3
+    assert bool((out[M] == 7.0).all())          # nothing past the last row
+
+
 @pytest.mark.parametrize("M,N,Kd,act", [(1, 4, 4, 0), (63, 36, 100, 1), (65, 516, 2052, 0), (129, 68, 64, 1),
                                         (64, 512, 2048, 0), (700, 2048, 96, 1), (1532, 512, 2048, 0), (3001, 260, 36, 1)])
 def test_linear_f32_splits(A, M, N, Kd, act):
