@@ -618,89 +618,120 @@ __global__ void __launch_bounds__(kSelThreads)
 
 // ---------------------------------------------------------------- Eq. 4 statistics
 constexpr int kStatThreads = 256;
+constexpr int kStatRows = 32;   // rows a block sums at a time
 
-// One warp per row: fp32 sums a.b, |a|^2, |b|^2; per block fixed-order fp64
-// sums of either the row cosines (TOKEN) or the three sums (FLAT).
+// The fp64 part of Eq. 4 for a block's kStatRows rows at once, one row a lane of
+// the first warp (sums: the rows' fp32 a.b, |a|^2, |b|^2): row cosines (TOKEN) or the
+// three sums (FLAT), added to the lane's acc. A square root or division in fp64
+// takes the SM hundreds of cycles a warp however few lanes need it: with a warp per
+// row, all lanes computing the same cosine, this bound the pass. With the fixed-order
+// sum behind it: 8192 x 2048 bf16 rows 27 -> 15 us, 32768 x 2048 80 -> 60 us; the
+// chunk partials of 8192 x 2048, 16.8 MB, 36 -> about 15 us.
+__device__ __forceinline__ void cos_rows32(const float (*sums)[3], int64_t r0, int64_t n_rows, int mode,
+                                           double (&acc)[3]) {
+  const int lane = threadIdx.x;
+  if (lane >= kStatRows || r0 + lane >= n_rows) return;
+  const float dot = sums[lane][0], na = sums[lane][1], nb = sums[lane][2];
+  if (mode == 0) {
+    const double den = fmax(sqrt((double)na), 1e-8) * fmax(sqrt((double)nb), 1e-8);
+    acc[0] += (double)dot / den;
+  } else {
+    acc[0] += dot; acc[1] += na; acc[2] += nb;
+  }
+}
+// The first warp's accumulators in a fixed order into the block's partial sums.
+__device__ __forceinline__ void cos_store(const double (&acc)[3], double* partials) {
+  if (threadIdx.x >= 32) return;
+  for (int j = 0; j < 3; ++j) {
+    const double s = warp_sum(acc[j]);
+    if (threadIdx.x == 0) partials[(int64_t)blockIdx.x * 3 + j] = s;
+  }
+}
+
+// Eq. 4 sums over rows: a warp takes four rows at once (fp32 sums a.b, |a|^2,
+// |b|^2), then the fp64 part over the block's 32 rows.
 template <typename T>
 __global__ void __launch_bounds__(kStatThreads) cos_rows_kernel(const T* a, const T* b,
                                                                 int64_t n_rows, int d, int mode,
                                                                 double* partials) {
   pdl_wait();
   pdl_trigger();
-  constexpr int V = Elem<T>::kVec;
-  __shared__ double red[kStatThreads / 32][3];
+  constexpr int V = Elem<T>::kVec, R = kStatRows / (kStatThreads / 32);
+  __shared__ float sums[kStatRows][3];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t nwarps = (int64_t)gridDim.x * (kStatThreads / 32);
-  double acc0 = 0, acc1 = 0, acc2 = 0;
-  for (int64_t r = (int64_t)blockIdx.x * (kStatThreads / 32) + w; r < n_rows; r += nwarps) {
-    float dot = 0.f, na = 0.f, nb = 0.f;
-    for (int c = lane * V; c < d; c += 32 * V) {
-      float fa[V], fb[V];
-      load_vec(a + r * d + c, fa);
-      load_vec(b + r * d + c, fb);
+  double acc[3] = {0, 0, 0};
+  for (int64_t r0 = (int64_t)blockIdx.x * kStatRows; r0 < n_rows; r0 += (int64_t)gridDim.x * kStatRows) {
+    float dot[R], na[R], nb[R];
 #pragma unroll
-      for (int j = 0; j < V; ++j) {
-        dot = fmaf(fa[j], fb[j], dot);
-        na = fmaf(fa[j], fa[j], na);
-        nb = fmaf(fb[j], fb[j], nb);
+    for (int i = 0; i < R; ++i) dot[i] = na[i] = nb[i] = 0.f;
+    for (int c = lane * V; c < d; c += 32 * V) {
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        const int64_t r = min(r0 + w * R + i, n_rows - 1);   // past the end: read again, left out below
+        float fa[V], fb[V];
+        load_vec(a + r * d + c, fa);
+        load_vec(b + r * d + c, fb);
+#pragma unroll
+        for (int j = 0; j < V; ++j) {
+          dot[i] = fmaf(fa[j], fb[j], dot[i]);
+          na[i] = fmaf(fa[j], fa[j], na[i]);
+          nb[i] = fmaf(fb[j], fb[j], nb[i]);
+        }
       }
     }
-    dot = warp_sum(dot);
-    na = warp_sum(na);
-    nb = warp_sum(nb);
-    if (mode == 0) {
-      const double den = fmax(sqrt((double)na), 1e-8) * fmax(sqrt((double)nb), 1e-8);
-      acc0 += (double)dot / den;
-    } else {
-      acc0 += dot; acc1 += na; acc2 += nb;
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      const float x = warp_sum(dot[i]), y = warp_sum(na[i]), z = warp_sum(nb[i]);
+      if (lane == 0) {
+        sums[w * R + i][0] = x;
+        sums[w * R + i][1] = y;
+        sums[w * R + i][2] = z;
+      }
     }
+    __syncthreads();
+    cos_rows32(sums, r0, n_rows, mode, acc);
+    __syncthreads();
   }
-  if (lane == 0) { red[w][0] = acc0; red[w][1] = acc1; red[w][2] = acc2; }
-  __syncthreads();
-  if (threadIdx.x < 3) {
-    double s = 0;
-    for (int i = 0; i < kStatThreads / 32; ++i) s += red[i][threadIdx.x];
-    partials[(int64_t)blockIdx.x * 3 + threadIdx.x] = s;
-  }
+  cos_store(acc, partials);
 }
 
 // Eq. 4 from per-chunk partials {a.b, |a|^2, |b|^2} ([n_rows][nch] float4,
-// written by a projection epilogue): one warp per row sums its chunks (fp32,
-// fixed lane order), then the same per-block fixed-order fp64 sums as
-// cos_rows_kernel.
-__global__ void __launch_bounds__(kStatThreads) cos_chunks_kernel(const float4* parts, int64_t n_rows,
-                                                                  int nch, int mode, double* partials) {
+// written by a projection epilogue): 16 lanes a row sum its chunks (fp32, fixed
+// order), then the fp64 part as in cos_rows_kernel.
+constexpr int kChunkThreads = 16 * kStatRows;
+__global__ void __launch_bounds__(kChunkThreads) cos_chunks_kernel(const float4* parts, int64_t n_rows,
+                                                                   int nch, int mode, double* partials) {
   pdl_wait();
   pdl_trigger();
-  __shared__ double red[kStatThreads / 32][3];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t nwarps = (int64_t)gridDim.x * (kStatThreads / 32);
-  double acc0 = 0, acc1 = 0, acc2 = 0;
-  for (int64_t r = (int64_t)blockIdx.x * (kStatThreads / 32) + w; r < n_rows; r += nwarps) {
-    float dot = 0.f, na = 0.f, nb = 0.f;
-    for (int c = lane; c < nch; c += 32) {
-      const float4 f = parts[r * nch + c];
-      dot += f.x;
-      na += f.y;
-      nb += f.z;
+  __shared__ float sums[kStatRows][3];
+  const int l16 = threadIdx.x & 15, row = threadIdx.x >> 4;
+  double acc[3] = {0, 0, 0};
+  for (int64_t r0 = (int64_t)blockIdx.x * kStatRows; r0 < n_rows; r0 += (int64_t)gridDim.x * kStatRows) {
+    float v[3] = {0.f, 0.f, 0.f};
+    if (r0 + row < n_rows) {
+      const float4* q = parts + (r0 + row) * nch;
+#pragma unroll 4
+      for (int c = l16; c < nch; c += 16) {
+        const float4 f = q[c];
+        v[0] += f.x;
+        v[1] += f.y;
+        v[2] += f.z;
+      }
     }
-    dot = warp_sum(dot);
-    na = warp_sum(na);
-    nb = warp_sum(nb);
-    if (mode == 0) {
-      const double den = fmax(sqrt((double)na), 1e-8) * fmax(sqrt((double)nb), 1e-8);
-      acc0 += (double)dot / den;
-    } else {
-      acc0 += dot; acc1 += na; acc2 += nb;
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) v[j] += __shfl_xor_sync(0xffffffffu, v[j], o);
+    if (l16 == 0) {
+      sums[row][0] = v[0];
+      sums[row][1] = v[1];
+      sums[row][2] = v[2];
     }
+    __syncthreads();
+    cos_rows32(sums, r0, n_rows, mode, acc);
+    __syncthreads();
   }
-  if (lane == 0) { red[w][0] = acc0; red[w][1] = acc1; red[w][2] = acc2; }
-  __syncthreads();
-  if (threadIdx.x < 3) {
-    double s = 0;
-    for (int i = 0; i < kStatThreads / 32; ++i) s += red[i][threadIdx.x];
-    partials[(int64_t)blockIdx.x * 3 + threadIdx.x] = s;
-  }
+  cos_store(acc, partials);
 }
 
 // Fixed-order sum of the per-block partials, added to acc.
@@ -1017,7 +1048,7 @@ cudaError_t select_gather_norm(int dtype, const float* scores, int B, int T, int
 // Fixed block count for a given row count (independent of the device), so the
 // fixed-order sums are reproducible everywhere.
 int stats_partials_count(int64_t n_rows) {
-  const int64_t want = (n_rows + (kStatThreads / 32) - 1) / (kStatThreads / 32);
+  const int64_t want = (n_rows + kStatRows - 1) / kStatRows;
   const int64_t cap = kStatMaxBlocks;
   return (int)(want < cap ? (want > 0 ? want : 1) : cap);
 }
@@ -1043,7 +1074,7 @@ cudaError_t cos_stats_chunks(const float4* parts, int64_t n_rows, int nch, int m
                              double* acc, const Dev& dev) {
   if (n_rows <= 0) return cudaSuccess;
   const int nb = stats_partials_count(n_rows);
-  cudaError_t e = launch_pdl(cos_chunks_kernel, dim3(nb), dim3(kStatThreads), 0, dev.stream, parts, n_rows, nch,
+  cudaError_t e = launch_pdl(cos_chunks_kernel, dim3(nb), dim3(kChunkThreads), 0, dev.stream, parts, n_rows, nch,
                              mode, partials);
   if (e != cudaSuccess) return e;
   return launch_pdl(cos_finish_kernel, dim3(1), dim3(256), 0, dev.stream, partials, nb, n_rows, mode, acc);

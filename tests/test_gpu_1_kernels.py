@@ -369,3 +369,23 @@ def test_layer_stats(A, n, d, dtype):
     A.adadsf_layer_stats(ad, bd, again)
     A.adadsf_layer_stats(ad, ad, again)
     assert again.cpu().numpy().tolist() == got.tolist()  # bit-reproducible
+
+
+@pytest.mark.parametrize("n,d,dtype", [(31, 8, "bf16"), (32, 264, "bf16"), (33, 4, "f32"), (70001, 72, "bf16")])
+def test_layer_stats_row_groups(A, n, d, dtype):
+    """Rows summed 32 at a time: last groups short, full and of one row, and more
+    groups than blocks. A row's fp32 sums hold d / 32 + 5 roundings at most, a
+    cosine three such sums, so well under 1e-5 each; the sum over rows is fp64."""
+    td = torch.bfloat16 if dtype == "bf16" else torch.float32
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    a = torch.randn((n, d), generator=gen, device="cuda").to(td)
+    b = (a.float() + 0.7 * torch.randn((n, d), generator=gen, device="cuda")).to(td)
+    acc = torch.zeros(2, dtype=torch.float64, device="cuda")
+    flat = torch.zeros(3, dtype=torch.float64, device="cuda")
+    A.adadsf_layer_stats(a, b, acc)
+    A.adadsf_layer_stats(a, b, flat, mode=A.STATS_FLAT)
+    a, b = a.double(), b.double()
+    dot, na, nb = (a * b).sum(1), (a * a).sum(1), (b * b).sum(1)
+    assert acc[1].item() == n
+    assert acc[0].item() == pytest.approx((dot / (na.sqrt() * nb.sqrt())).sum().item(), rel=1e-5)
+    assert flat.tolist() == pytest.approx([dot.sum().item(), na.sum().item(), nb.sum().item()], rel=1e-5)
