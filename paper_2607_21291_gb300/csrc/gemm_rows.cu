@@ -14,9 +14,9 @@
 // they come. The warps' sums are added in warp order through shared memory
 // (bit-reproducible), and the next tile's first pieces load meanwhile.
 //
-// The line to the tensor-core kernels lies at the weights' size (MB), 28 up to 8 rows
-// and 16 above, because those stream large weights faster (TMA boxes keep more in
-// flight than 16 loads a lane). us per product from a cold L2, there / here:
+// Its line lies at the weights' size (MB), 28 up to 8 rows and 16 above: larger
+// weights stream faster by TMA, whose boxes keep more in flight than 16 loads a lane (the second
+// kernel below, or the tensor-core kernels). us per product from a cold L2, there / here:
 //   N x K            MB     1 row          16 rows
 //   768 x 768        1.2    5.3 / 2.1      5.1 / 2.9
 //   2304 x 768       3.5    5.4 / 2.5      5.4 / 3.2
@@ -216,6 +216,199 @@ __global__ void __launch_bounds__(kGrThreads, 1)
   }
 }
 
+// ---------------------------------------------------------------- larger weights
+constexpr int kGsWarps = 8;           // consumer warps; one 16-k product of a stage each
+constexpr int kGsThreads = 32 * (kGsWarps + 1);
+constexpr int kGsGroups = 8;          // 8-row groups of W a tile takes
+constexpr int kGsBox = 2048;          // bytes of 8 rows x 128 k
+constexpr int kGsMaxStages = 12;
+constexpr int kGsRingBytes = 184 * 1024;
+
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const void* tmap, int c0, int c1, int c2, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(tmap)), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
+      : "memory");
+}
+__device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+__device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+
+// Past the line of the kernel above a product streams through TMA. Against the
+// tensor-core kernels, whose tiles of 128 weight rows and splits of 2 or 4 fill 112 to
+// 144 of the SMs, the groups divide over pairs of CTAs, each CTA half of K, so
+// that every SM streams and only one partial tile passes between two CTAs. A thread
+// brings stages of 128 k, one box of W (a tile's rows, two blocks of 128-byte swizzled
+// rows) and one of A, into a ring of 170 KB; each of eight warps takes one 16-k product of a
+// stage (mma.sync: 24 of them a stage at 48 rows, far from a limit). The sums
+// of the warps are added in warp order, the pair's halves exchange theirs and
+// each finishes half of the outputs. One box of 8 rows each instead of one a stage: 47 us
+// at 3584 x 18944, TMA-issue bound, to 29. Chains of products of different weights, us
+// each at 16 rows, tensor-core kernels / here: 3584 x 18944 29.2 / 26.0, 4608 x 3584
+// 10.5 / 9.5, 2048 x 8192 12.9 / 13.0, 3584 x 3584 9.5 / 9.3, 4864 x 2048 8.4 / 7.8; 16
+// sequences at the Qwen2.5-7B shape, two layers, 16 steps 4241 -> 4084 us. With
+// more rows than one tile of 64 a pair (N > 4864) the exchanges and the repeated rows of A
+// lose: 8192 x 2048 12.5 / 14.5, 18944 x 3584 29 / 37, which stay where they were.
+// tmW2 / tmX2: the second K source.
+template <int NT>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGsThreads, 1)
+    gemm_rows_stream_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
+                            const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUtensorMap tmX2,
+                            const __grid_constant__ RowsDev p, int U, int S, int* err,
+                            unsigned long long timeout_ns) {
+  constexpr int NC = NT * 8;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  __shared__ uint64_t bars[2 * kGsMaxStages + 1];
+  __shared__ int abort_s;
+  volatile int* abort_flag = &abort_s;
+  const int pairs = (U + 1) / 2;
+  const uint32_t stage_bytes = (uint32_t)(U + NT) * kGsBox;
+  float* red = reinterpret_cast<float*>(smem + (size_t)S * stage_bytes);   // [warp][pair][16][NC]
+  float* recv = red + kGsWarps * pairs * 16 * NC;                          // [pairs * 8 * NC]: from the peer
+  const uint32_t ring = smem_u32(smem), full0 = smem_u32(bars), empty0 = full0 + 8 * kGsMaxStages,
+                 rbar = empty0 + 8 * kGsMaxStages;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = (int)cluster_ctarank();
+  const int cl = blockIdx.x >> 1, ncl = gridDim.x >> 1;
+  // this pair's groups [lo, lo + cnt), cnt <= U, and this CTA's stages [k0, k1), n1 of all from the first source
+  const int lo = (int)((int64_t)p.groups * cl / ncl), cnt = (int)((int64_t)p.groups * (cl + 1) / ncl) - lo;
+  const int n1 = (p.n1 + 3) / 4, n = n1 + (p.n - p.n1 + 3) / 4;
+  const int k0 = rank == 0 ? 0 : n / 2, k1 = rank == 0 ? n / 2 : n;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < S; ++s) {
+      mbar_init(full0 + 8 * s, 1);
+      mbar_init(empty0 + 8 * s, kGsWarps);
+    }
+    mbar_init(rbar, kGsWarps);
+    abort_s = 0;
+    fence_barrier_init();
+  }
+  cluster_sync();   // the peer's arrivals find the barriers initialised
+
+  if (warp == kGsWarps) {
+    if (lane == 0) {
+      tma_prefetch_desc(&tmW);
+      tma_prefetch_desc(&tmX);
+      int stage = 0;
+      uint32_t phase = 0;
+      int64_t issued = 0;
+      auto load_w = [&](int k, int s) {
+        const bool s2 = k >= n1;
+        mbar_arrive_expect_tx(full0 + 8 * s, stage_bytes);
+        tma_load_3d(ring + s * stage_bytes, s2 ? &tmW2 : &tmW, 0, lo * 8, 2 * (s2 ? k - n1 : k), full0 + 8 * s);
+      };
+      auto load_x = [&](int k, int s) {
+        const bool s2 = k >= n1;
+        tma_load_3d(ring + s * stage_bytes + U * kGsBox, s2 ? &tmX2 : &tmX, 0, 0, 2 * (s2 ? k - n1 : k), full0 + 8 * s);
+      };
+      // the weights of the first stages do not depend on the kernel before
+      const int pre = min(S, k1 - k0);
+      for (int i = 0; i < pre; ++i) load_w(k0 + i, i);
+      pdl_wait();
+      for (int k = k0; k < k1; ++k) {
+        if (k - k0 >= pre) {
+          if (!mbar_wait_bounded(empty0 + 8 * stage, phase ^ 1, abort_flag, err, timeout_ns)) break;
+          load_w(k, stage);
+        }
+        load_x(k, stage);
+        ++issued;
+        if (++stage == S) { stage = 0; phase ^= 1; }
+      }
+      pdl_trigger();
+      for (int s = 0; s < S && s < issued; ++s) {   // every copy has landed before the block goes
+        const int64_t last = s + ((issued - 1 - s) / S) * S;
+        mbar_wait_drain(full0 + 8 * s, (uint32_t)((last / S) & 1), timeout_ns);
+      }
+    }
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  } else {
+    pdl_wait();
+    // this warp's product of a stage: 16-byte columns ck and ck + 1 of the stage's column kb
+    const int kb = warp >> 2, ck = (warp & 3) * 2;
+    const int wr = (lane & 7) + ((lane >> 3) & 1) * 8;   // ldmatrix row of W: two groups
+    const uint32_t w_at = (uint32_t)(kb * U * 1024 + wr * 128 + (((ck + (lane >> 4)) ^ (wr & 7)) << 4));
+    const int xr = (lane & 7) + (NT == 2 ? (lane >> 4) * 8 : 0);
+    const uint32_t x_at = (uint32_t)(U * kGsBox + kb * 1024 * NT + xr * 128 + (((ck + ((lane >> 3) & 1)) ^ (xr & 7)) << 4));
+    const int gid = lane >> 2, tig = lane & 3;
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;   // after a wait that ran out the warps go on without waiting, to the end
+    float acc[kGsGroups / 2][NT][4];
+#pragma unroll
+    for (int q = 0; q < kGsGroups / 2; ++q)
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt) acc[q][nt][0] = acc[q][nt][1] = acc[q][nt][2] = acc[q][nt][3] = 0.f;
+    for (int k = k0; k < k1; ++k) {
+      ok = __all_sync(~0u, mbar_wait_bounded(full0 + 8 * stage, phase, abort_flag, err, timeout_ns));
+      if (!ok) break;
+      const uint32_t base = ring + stage * stage_bytes;
+      uint32_t xv[4];
+      ldmatrix_x4(xv, base + x_at);
+#pragma unroll
+      for (int q = 0; q < kGsGroups / 2; ++q) {
+        if (2 * q < cnt) {   // with an odd count the last 8 rows are others' bytes: their sums are dropped
+          uint32_t wv[4];
+          ldmatrix_x4(wv, base + q * 2 * 1024 + w_at);
+#pragma unroll
+          for (int nt = 0; nt < NT; ++nt)
+            mma_rows(acc[q][nt], wv[0], wv[1], wv[2], wv[3], xv[2 * nt], xv[2 * nt + 1]);
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(empty0 + 8 * stage);
+      if (++stage == S) { stage = 0; phase ^= 1; }
+    }
+    float* mine = red + warp * pairs * 16 * NC;
+#pragma unroll
+    for (int q = 0; q < kGsGroups / 2; ++q) {
+      if (2 * q < cnt) {
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+          float* d = mine + (q * 16 + gid) * NC + nt * 8 + tig * 2;
+          *reinterpret_cast<float2*>(d) = make_float2(acc[q][nt][0], acc[q][nt][1]);
+          *reinterpret_cast<float2*>(d + 8 * NC) = make_float2(acc[q][nt][2], acc[q][nt][3]);
+        }
+      }
+    }
+    named_bar_sync(1, kGsWarps * 32);
+    // the peer's half of the outputs goes to the peer, then this CTA's half is finished
+    const int half = cnt * 4 * NC;
+    const uint32_t to = map_to_cta(smem_u32(recv), (uint32_t)(rank ^ 1));
+    for (int o = threadIdx.x; o < half; o += kGsWarps * 32) {
+      float v = 0.f;
+#pragma unroll
+      for (int w = 0; w < kGsWarps; ++w) v += red[w * pairs * 16 * NC + (rank ^ 1) * half + o];
+      st_cluster_f32(to + 4 * o, v);
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive_cluster(map_to_cta(rbar, (uint32_t)(rank ^ 1)));
+    if (ok) mbar_wait_bounded(rbar, 0, abort_flag, err, timeout_ns);
+    asm volatile("fence.acq_rel.cluster;" ::: "memory");
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    for (int o = threadIdx.x; o < half; o += kGsWarps * 32) {
+      float v = 0.f;
+#pragma unroll
+      for (int w = 0; w < kGsWarps; ++w) v += red[w * pairs * 16 * NC + rank * half + o];
+      const int e = rank * half + o, m = e % NC;
+      if (m < p.M) rows_epilogue<false>(p, m, lo * 8 + e / NC, v + recv[o], 0.f);
+    }
+  }
+  __syncwarp();
+  // the peer has written its sums here before this CTA's memory goes
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 bool rows_dev(const GemmArgs& a, RowsDev& p) {
   p = RowsDev{};
   if (a.M <= 0 || a.M > kGrMaxRows || a.N % 8 || a.K % 32 || a.K2 % 32 || a.a_gather) return false;
@@ -254,21 +447,56 @@ bool rows_dev(const GemmArgs& a, RowsDev& p) {
   return true;
 }
 
+double weight_bytes(const GemmArgs& g) {
+  return 2.0 * g.N * ((double)(g.epi.act == ACT_SWIGLU ? 2 : 1) * g.K + (g.K2 > 0 ? g.K2 : 0));
+}
+
+// Weights (bytes) up to which the first kernel is the faster one.
+double rows_line(const GemmArgs& a) { return a.M <= 8 ? 28e6 : 16e6; }
+
+// Products for the streaming kernel: more weights than that, one tile a pair of CTAs. From
+// 512 columns on it is the faster one (512 x 20480 23.4 us by the tensor-core kernels, 22.7 here);
+// below, too few pairs of CTAs have a group.
+bool streams(const GemmArgs& a, int num_sms) {
+  return a.epi.act != ACT_SWIGLU && a.K % 64 == 0 && a.K2 % 64 == 0 && a.N >= 512 &&
+         a.N / 8 <= kGsGroups * (num_sms / 2) &&
+         weight_bytes(a) > rows_line(a);
+}
+
+template <int NT>
+cudaError_t launch_stream(const GemmArgs& a, const RowsDev& p, const Dev& dev) {
+  const int ncl = std::min(dev.num_sms / 2, p.groups);
+  const int U = (p.groups + ncl - 1) / ncl, pairs = (U + 1) / 2;
+  CUtensorMap w, x, w2, x2;
+  auto map = [](CUtensorMap* m, const void* ptr, int64_t rows, int k, int64_t ld, int box_rows) {
+    return make_tmap_bf16_k(m, ptr, (uint64_t)rows, (uint64_t)k, (uint64_t)ld, (uint32_t)box_rows);
+  };
+  if (!map(&w, a.W, a.N, a.K, a.ldw, 8 * U) || !map(&x, a.A, a.M, a.K, a.lda, 8 * NT)) return cudaErrorInvalidValue;
+  w2 = w;
+  x2 = x;
+  if (a.K2 > 0 && (!map(&w2, a.Wk2, a.N, a.K2, a.ldwk2, 8 * U) || !map(&x2, a.A2, a.M, a.K2, a.lda2, 8 * NT)))
+    return cudaErrorInvalidValue;
+  const int stage = (U + NT) * kGsBox, S = std::min(kGsMaxStages, kGsRingBytes / stage);
+  const int smem = 1024 + S * stage + (kGsWarps * pairs * 16 + pairs * 8) * NT * 8 * 4;
+  const cudaError_t e = allow_smem(gemm_rows_stream_kernel<NT>, smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(gemm_rows_stream_kernel<NT>, dim3((unsigned)(2 * ncl)), dim3(kGsThreads), (size_t)smem, dev.stream, w,
+                    x, w2, x2, p, U, S, dev.err, kWaitTimeoutNs);
+}
+
 }  // namespace
 
-bool gemm_rows_takes(const GemmArgs& a, const GemmArgs* b) {
+bool gemm_rows_takes(const GemmArgs& a, const GemmArgs* b, int num_sms) {
   RowsDev p;
   if (!rows_dev(a, p) || (b && !rows_dev(*b, p))) return false;
   if (b && (a.epi.act == ACT_SWIGLU || b->epi.act == ACT_SWIGLU || a.M != b->M)) return false;
-  auto bytes = [](const GemmArgs& g) {
-    return 2.0 * g.N * ((double)(g.epi.act == ACT_SWIGLU ? 2 : 1) * g.K + (g.K2 > 0 ? g.K2 : 0));
-  };
-  return bytes(a) + (b ? bytes(*b) : 0.0) <= (a.M <= 8 ? 28e6 : 16e6);
+  return weight_bytes(a) + (b ? weight_bytes(*b) : 0.0) <= rows_line(a) || (!b && streams(a, num_sms));
 }
 
 cudaError_t gemm_rows(const GemmArgs& a, const GemmArgs* b, const Dev& dev) {
   RowsDev p, q = {};
   if (!rows_dev(a, p) || (b && !rows_dev(*b, q))) return cudaErrorInvalidValue;
+  if (!b && streams(a, dev.num_sms)) return a.M <= 8 ? launch_stream<1>(a, p, dev) : launch_stream<2>(a, p, dev);
   const dim3 grid((unsigned)std::min(dev.num_sms, p.groups + q.groups)), block(kGrThreads);
   if (a.epi.act == ACT_SWIGLU)
     return a.M <= 8 ? launch_pdl(gemm_rows_kernel<1, true>, grid, block, 0, dev.stream, p, q)

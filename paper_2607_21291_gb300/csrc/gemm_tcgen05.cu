@@ -1378,6 +1378,20 @@ bool make_tmap_bf16(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t col
   return r == CUDA_SUCCESS;
 }
 
+// The same matrix as [cols / 64][rows][64] (cols a multiple of 64): a box brings
+// 128 k of box_rows rows as two blocks of 128-byte rows.
+bool make_tmap_bf16_k(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols, uint64_t ld, uint32_t box_rows) {
+  auto fn = encode_fn();
+  if (!fn || cols % 64) return false;
+  cuuint64_t dims[3] = {64, rows, cols / 64};
+  cuuint64_t strides[2] = {ld * 2, 128};
+  cuuint32_t box[3] = {64, box_rows, 2};
+  cuuint32_t estr[3] = {1, 1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 namespace {
 
 bool make_tmap(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols, uint64_t ld,
@@ -1739,7 +1753,7 @@ size_t gemm_split_scratch_bytes() { return (size_t)160 * BM * 256 * 4; }
 cudaError_t gemm_bf16(const GemmArgs& a, const Dev& dev) {
   if (a.M <= 0) return cudaSuccess;
   if (a.a_gather && (a.epi.act == ACT_SWIGLU || a.a_gather_rows <= 0)) return cudaErrorInvalidValue;
-  if (gemm_rows_takes(a, nullptr)) return gemm_rows(a, nullptr, dev);
+  if (gemm_rows_takes(a, nullptr, dev.num_sms)) return gemm_rows(a, nullptr, dev);
   // SwiGLU: 256 x 128 gate/up tiles on CTA pairs when that still gives every
   // pair of SMs at least two tiles.
   if (a.epi.act == ACT_SWIGLU) {
@@ -1760,7 +1774,7 @@ cudaError_t gemm_bf16_grouped(const GemmArgs& a, const GemmArgs& b, const Dev& d
     return g.epi.act != ACT_SWIGLU && g.K2 == 0;
   };
   if (!plain(a) || !plain(b)) return cudaErrorInvalidValue;
-  if (gemm_rows_takes(a, &b)) return gemm_rows(a, &b, dev);
+  if (gemm_rows_takes(a, &b, dev.num_sms)) return gemm_rows(a, &b, dev);
   // Fewest rounds of tiles (a k-block costs the same for any tile width);
   // ties go to CTA pairs (half the weight bytes per SM), then to 256-wide
   // tiles. Problem `a` comes first in the tile order: pass the one with the

@@ -119,15 +119,17 @@ struct Dev {
 // elements), box_cols x box_rows boxes, 128-byte swizzle, zero fill.
 bool make_tmap_bf16(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols, uint64_t ld,
                     uint32_t box_cols, uint32_t box_rows);
+// The same with 64-column blocks as a third dimension, two of them a box.
+bool make_tmap_bf16_k(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols, uint64_t ld, uint32_t box_rows);
 
 // gemm_tcgen05.cu -- bf16 tensor-core projections (tcgen05 + TMEM + TMA).
 cudaError_t gemm_bf16(const GemmArgs& a, const Dev& dev);
 // Two independent plain projections (no SwiGLU, router or second K source)
 // in one launch.
 cudaError_t gemm_bf16_grouped(const GemmArgs& a, const GemmArgs& b, const Dev& dev);
-// gemm_rows.cu -- bf16 projections of at most 16 rows and few weights (b: a second
-// problem on the same number of rows, or null).
-bool gemm_rows_takes(const GemmArgs& a, const GemmArgs* b);
+// gemm_rows.cu -- bf16 projections of at most 16 rows with few weights or few columns
+// (b: a second problem on the same number of rows, or null).
+bool gemm_rows_takes(const GemmArgs& a, const GemmArgs* b, int num_sms);
 cudaError_t gemm_rows(const GemmArgs& a, const GemmArgs* b, const Dev& dev);
 // train.cu -- alignment objective (Eqs. 9-10) and the router gradient.
 int train_row_blocks(int64_t n);

@@ -166,6 +166,30 @@ def test_linear_bf16_few_rows(A, M, N, Kd, act):
     assert bool((out[M] == 7.0).all())          # nothing past the last row
 
 
+@pytest.mark.parametrize("M,N,Kd,act", [(1, 3584, 4096, 0), (8, 3584, 3968, 1), (9, 1088, 8256, 0), (16, 4864, 1728, 1),
+                                        (16, 4928, 1728, 0), (13, 512, 16448, 0), (16, 448, 20480, 0)])
+def test_linear_bf16_few_rows_streamed(A, M, N, Kd, act):
+    """At most 16 rows and more weights than the direct kernel takes: one and two
+    8-row halves, 1 to 8 groups of columns a pair of CTAs, K of an odd number of 64-element
+    blocks (and N past either end of the range, the tensor-core kernels). One bf16
+    rounding of the output (2^-9 of an element, under 8e-3 of the largest)."""
+    g = torch.Generator(device="cuda").manual_seed(N + Kd)
+    rnd = lambda *shape: torch.randn(shape, generator=g, device="cuda")
+    x, w, b = rnd(M, Kd).bfloat16(), (rnd(N, Kd) / Kd ** 0.5).bfloat16(), rnd(N).bfloat16()
+    out = torch.full((M + 1, N), 7.0, dtype=torch.bfloat16, device="cuda")
+    ws = A.workspace(A.LINEAR_SPLIT_WS_BYTES)
+    A.adadsf_linear(x, w, b, out[:M], act=act, ws=ws)
+    assert A.adadsf_sync_check(ws) == A.OK
+    ref = x.double() @ w.double().T + b.double()
+    if act:
+        ref = torch.nn.functional.gelu(ref)
+    assert H.max_rel(H.to_np(out[:M]), ref.cpu().numpy()) < 8e-3
+    assert bool((out[M] == 7.0).all())          # nothing past the last row
+    again = torch.empty_like(out[:M])
+    A.adadsf_linear(x, w, b, again, act=act, ws=ws)
+    assert torch.equal(again, out[:M])
+
+
 @pytest.mark.parametrize("M,N,Kd,act", [(1, 4, 4, 0), (63, 36, 100, 1), (65, 516, 2052, 0), (129, 68, 64, 1),
                                         (64, 512, 2048, 0), (700, 2048, 96, 1), (1532, 512, 2048, 0), (3001, 260, 36, 1)])
 def test_linear_f32_splits(A, M, N, Kd, act):

@@ -27,6 +27,7 @@ def A():
 
 QWEN_SMALL = S.QWEN25_1_5B.replace(d=1024, n_heads=8, n_kv_heads=2, ffn=1536, n_layers=3, vocab=500)
 NEOX_SMALL = S.PYTHIA_160M.replace(n_layers=3, vocab=500)
+NEOX_WIDE = S.PYTHIA_1_4B.replace(n_layers=1, vocab=500)
 NEOX_F32 = S.PYTHIA_70M.replace(n_layers=2, vocab=500)
 # the Qwen2.5-7B attention geometry (28 query heads on 4 key/value heads,
 # head_dim 128) with a narrow MLP: caches of several hundred keys spread over
@@ -52,6 +53,9 @@ CASES = [
     (NEOX_SMALL, 17, 40, [20, 40, 13], 3, 48, False, None),
     (NEOX_SMALL, 9, 33, [20, 33, 13], 3, 40, False, None),
     (QWEN_G16, 2, 700, [500, 700], 3, 720, False, H.BF16_DEEP_ELEM_TOL),
+    # output and MLP-down projections of 42 MB, streamed in one sum
+    (NEOX_WIDE, 2, 40, [20], 2, 48, False, None),
+    (NEOX_WIDE, 9, 20, [13], 2, 24, True, None),
 ]
 
 
