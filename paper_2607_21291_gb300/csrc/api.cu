@@ -451,11 +451,17 @@ adadsf_status layer_impl(const adadsf_model_cfg* c, const adadsf_layer_weights* 
     rows = dec->rows;
     pos = dec->pos;
   } else if (!dense) {
-    if (M <= 32LL * dev.num_sms) {
-      // a3 + a4: Top-K of each sequence fused with the gather of the kept rows
-      // and their norms (NeoX: LN1 and LN2 of the same row). Every block
-      // repeats its sequence's selection: worth it while a launch less
-      // outweighs that (up to about one row per warp on four blocks per SM).
+    // a3 + a4: Top-K of each sequence fused with the gather of the kept rows and
+    // their norms (NeoX: LN1 and LN2 of the same row). Every block repeats its
+    // sequence's selection and normalises a row a warp: worth it while a launch
+    // less outweighs that, on sequences below 2048 and 4 MB of kept rows, and
+    // rows below 4 KB or sequences below 512. A layer by it / by two launches, half kept, us:
+    // d 768 B 8 T 256 51.0 / 52.8, B 4 T 1024 78.6 / 79.3, B 1 T 4096 112.9 / 107.2; d 1536 B 4 T 512
+    // 128.9 / 129.5, B 8 T 512 191 / 186, B 1 T 4096 240 / 223; d 2048 B 1 T 256
+    // 64.3 / 64.4, T 512 80.1 / 77.9, B 4 T 1024 180 / 170; fp32 d 512 B 4 T 256 123.7 / 125.4, B 1 T
+    // 4096 670 / 662.
+    const double row_bytes = (double)d * es;
+    if (M <= 32LL * dev.num_sms && T < 2048 && M * row_bytes < 4e6 && (row_bytes < 4096 || T < 512)) {
       TRY(launch(dev, ADADSF_KERNEL_TOPK_GATHER_NORM, false, 0,
                  BT * 4.0 + M * 8.0 + Md * es * (neox ? 3 : 2),
                  CALL(select_gather_norm(dt, lb.scores, B, T, K, x, d, !neox, w->ln1_w, w->ln1_b,

@@ -75,6 +75,18 @@ def test_sparse_layer(A, shape, B, T, K):
                            hx[b, skip].view(torch.int16 if shape.dtype == "bf16" else torch.int32))
 
 
+@pytest.mark.parametrize("shape,B,T,K,fused", [
+    (S.PYTHIA_160M, 1, 2047, 300, True), (S.PYTHIA_160M, 1, 2048, 300, False),
+    (S.PYTHIA_70M, 2, 2047, 65, True), (S.PYTHIA_70M, 2, 2048, 65, False),
+    (QWEN_SMALL, 2, 1000, 976, True), (QWEN_SMALL, 2, 1000, 977, False),
+    (S.PYTHIA_1_4B.replace(ffn=512), 1, 511, 33, True), (S.PYTHIA_1_4B.replace(ffn=512), 1, 512, 33, False)])
+def test_selection_launches(A, shape, B, T, K, fused):
+    """Each side of the lines between one launch for Top-K, gather and norm and
+    two: sequence length, bytes of kept rows, bytes of a row."""
+    kinds = _kinds(A, lambda: test_sparse_layer(A, shape, B, T, K))
+    assert ("topk_gather_norm" in kinds) == fused and ("topk" in kinds) != fused, kinds
+
+
 @pytest.mark.parametrize("shape", [S.PYTHIA_70M, S.PYTHIA_160M, QWEN_SMALL])
 def test_r1_is_dense_and_r0_identity(A, shape):
     B, T = 2, 96
