@@ -242,6 +242,9 @@ struct DecodeFront {
   int C_max;
   int32_t *lens, *rows, *pos, *kept_out;
 };
+// Router scores of few tokens (bf16, 64 hidden units).
+cudaError_t router_rows16(const void* x, int64_t n_rows, int d, const void* w1, const void* b1, const void* w2,
+                          const void* b2, float* scores, const Dev& dev);
 bool decode_front_fits(int dtype, int B, int h);
 cudaError_t decode_front(const DecodeFront& a, bool is_rms, const Dev& dev);
 // Set in pos[b] beside the position: the new token is counted in the layer's cache

@@ -480,6 +480,8 @@ cudaError_t router_tc(const void* x, int64_t rows, int d, const void* w1, const 
                       const void* b2, float* scores, float* tsq, int* sync, float* partials, const Dev& dev) {
   if (rows <= 0) return cudaSuccess;
   if (d % kRK != 0 || d <= 0) return cudaErrorInvalidValue;
+  // few tokens: rowwise.cu has both sides' times
+  if (!tsq && rows <= 16 * (int64_t)dev.num_sms) return router_rows16(x, rows, d, w1, b1, w2, b2, scores, dev);
   const int64_t n_tiles = (rows + kRM - 1) / kRM;
   const int nkb = d / kRK;
   RouterDev p{};

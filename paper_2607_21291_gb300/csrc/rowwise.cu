@@ -292,6 +292,60 @@ __global__ void __launch_bounds__(kRrThreads)
   cluster_sync();   // the eighths stay until the first CTA has read them
 }
 
+// Router scores of few tokens (bf16): a cluster of C CTAs takes 16 tokens, each CTA a
+// share of the features, as the launch above does, so that a few hundred tokens keep
+// every SM loading. The tensor-core kernel gives a CTA 128 tokens and all of d, whose
+// tiles arrive one after another: bound by what one SM loads (0.3 MB at d = 1024)
+// on 7 SMs at 777 tokens. us, that / this (in a graph, with 6.4 us of it or less for
+// an empty launch), 777 tokens and 2048:
+//   d 768 10.4 / 8.4, 10.4 / 8.4   d 1536 14.2 / 8.4, 14.4 / 10.4
+//   d 2048 13.0 / 8.4, 12.6 / 10.4   d 3584 14.6 / 10.4, 14.6 / 12.5
+// C is the largest that leaves all CTAs resident (two an SM); one more doubling
+// took 12.4 us at 777 tokens of d 1536. From more than 16 tokens an SM on (C = 1) it is
+// no faster: 4096 tokens 10.5 against 10.4 us at d 768, 18.6 against 14.5 at 3584.
+// Error against 64 bits 1.2e-7 (5.6e-7 to 1.9e-6 there).
+__global__ void __launch_bounds__(kRrThreads)
+    router_rows16_kernel(const bf16* x, int64_t n_rows, int d, const bf16* w1, const bf16* rb1, const bf16* w2,
+                         const bf16* rb2, float* scores) {
+  extern __shared__ __align__(16) uint8_t smem_r16[];
+  float* red = reinterpret_cast<float*>(smem_r16);                       // [warp][16][64]
+  float* part = red + RouterRows<bf16>::RED_FLOATS;                     // [16][64]: this CTA's share
+  const int C = (int)cluster_nctarank(), rank = (int)cluster_ctarank();
+  const int64_t r0 = (int64_t)(blockIdx.x / C) * kRrRows;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int n = d / 32;                                                 // pieces of 32 features
+  const int c_lo = n * rank / C, c_hi = n * (rank + 1) / C;
+  RouterPiece pc;
+  if (c_lo + warp < c_hi) pc.load_w(w1, d, c_lo + warp);                // weights: independent of the previous kernel
+  pdl_wait();
+  pdl_trigger();
+  const int64_t ra = min(r0 + (lane >> 2), n_rows - 1), rb = min(r0 + 8 + (lane >> 2), n_rows - 1);
+  const float4 u4 = router_rows_partial(x + ra * d, x + rb * d, w1, d, c_lo, c_hi, pc, red);
+  const int row = threadIdx.x >> 4, j0 = (threadIdx.x & 15) * 4;
+  *reinterpret_cast<float4*>(part + row * kRrUnits + j0) = u4;
+  cluster_sync();
+  if (rank == 0) {
+    const uint32_t at = smem_u32(part + row * kRrUnits + j0);
+    float u[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int q = 0; q < C; ++q) {
+      const float4 f = ld_cluster_f32x4(map_to_cta(at, q));
+      u[0] += f.x;
+      u[1] += f.y;
+      u[2] += f.z;
+      u[3] += f.w;
+    }
+    float s = 0.f;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float v = u[e] + __bfloat162float(rb1[j0 + e]);
+      s += __bfloat162float(w2[j0 + e]) * (v / (1.f + expf(-v)));
+    }
+    s = row16_sum(s);
+    if ((threadIdx.x & 15) == 0 && r0 + row < n_rows) scores[r0 + row] = s + __bfloat162float(rb2[0]);
+  }
+  cluster_sync();   // the shares stay until the first CTA has read them
+}
+
 // ---------------------------------------------------------------- TMA-staged gather + norm
 // For large row counts (HBM bound): one warp streams whole source rows into a
 // shared-memory ring with one bulk copy each (cp.async.bulk, completion on the
@@ -1043,6 +1097,22 @@ cudaError_t select_gather_norm(int dtype, const float* scores, int B, int T, int
                                                     out1, out2, idx, rows, dev)
                 : select_gather_norm_t<float, false>(scores, B, T, K, x, d, g1, b1, g2, b2, eps,
                                                      out1, out2, idx, rows, dev);
+}
+
+cudaError_t router_rows16(const void* x, int64_t n_rows, int d, const void* w1, const void* b1, const void* w2,
+                          const void* b2, float* scores, const Dev& dev) {
+  if (n_rows <= 0) return cudaSuccess;
+  const int64_t tiles = (n_rows + kRrRows - 1) / kRrRows;
+  if (tiles * 2 > 2 * (int64_t)dev.num_sms) return cudaErrorInvalidValue;
+  int C = 8;
+  while (C > 1 && tiles * C > 2 * dev.num_sms) C /= 2;
+  constexpr int smem = (RouterRows<bf16>::RED_FLOATS + kRrRows * kRrUnits) * 4;
+  const cudaError_t e = allow_smem(router_rows16_kernel, smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl_cluster(router_rows16_kernel, dim3((unsigned)(tiles * C)), dim3(kRrThreads), (size_t)smem, dev.stream,
+                            C, static_cast<const bf16*>(x), n_rows, d, static_cast<const bf16*>(w1),
+                            static_cast<const bf16*>(b1), static_cast<const bf16*>(w2), static_cast<const bf16*>(b2),
+                            scores);
 }
 
 // Fixed block count for a given row count (independent of the device), so the

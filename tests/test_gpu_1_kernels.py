@@ -224,6 +224,28 @@ def test_router_f32_edges(A, n, d, h):
     assert float(sc[n]) == 7.0
 
 
+@pytest.mark.parametrize("per_sm,off,d", [(0, 1, 64), (0, 15, 3584), (0, 17, 192), (4, 0, 1536), (4, 1, 1536),
+                                          (8, -3, 768), (8, 1, 768), (16, 0, 2048), (16, 1, 2048)])
+def test_router_few_tokens(A, per_sm, off, d):
+    """bf16 scores around the 16-token blocks, every cluster width (8, 4 and 2 CTAs
+    take up to 4, 8 and 16 tokens an SM), widths with fewer 32-feature pieces than
+    CTAs, and past the last width the 128-token tiles. Products are exact; an fp32
+    sum of d, then of 64 units: under 1e-5 of the scores' rms (2e-6 in rms measured
+    for the tiles)."""
+    n = per_sm * torch.cuda.get_device_properties(0).multi_processor_count + off
+    shape = S.PYTHIA_160M.replace(d=d, n_layers=1)
+    W = H.host_layer(shape, n + d)
+    x = S.round_to(S.hidden(n, 1, n, d)[0], "bf16")
+    outs = []
+    for _ in range(2):
+        sc = torch.full((n + 1,), 7.0, device="cuda")
+        A.adadsf_router_scores(A.make_cfg(shape), A.to_device(W, torch.bfloat16), H.to_dev(x, torch.bfloat16), sc[:n])
+        outs.append(sc.cpu())
+    ref = O.router_scores(x.astype(np.float64), H.f64(W))
+    assert H.elem_rel(outs[0][:n].numpy(), ref) < 1e-5
+    assert float(outs[0][n]) == 7.0 and torch.equal(*outs)
+
+
 @pytest.mark.parametrize("shape,n", [(S.PYTHIA_160M, 1), (S.PYTHIA_160M, 2048), (S.QWEN25_1_5B, 333),
                                      (S.PYTHIA_70M, 128), (S.PYTHIA_160M, 777), (S.PYTHIA_1_4B, 16384)])
 def test_router(A, shape, n):
