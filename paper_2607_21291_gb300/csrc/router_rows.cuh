@@ -31,7 +31,7 @@ struct RouterRows {
   static constexpr int RED_FLOATS = kRrWarps * kRrRows * kRrUnits;
   static constexpr int SMEM_FLOATS = kRrWarps * WARP_FLOATS > RED_FLOATS ? kRrWarps * WARP_FLOATS : RED_FLOATS;
   static constexpr int SMEM_BYTES = SMEM_FLOATS * 4;
-  static constexpr int MMA_BYTES = RED_FLOATS * 4;         // router_rows_units_mma
+  static constexpr int MMA_BYTES = RED_FLOATS * 4;         // router_rows_partial
 };
 
 // u[row][unit] (no bias) of 4 consecutive units: thread t holds row t / 16 and
@@ -137,7 +137,6 @@ __device__ __forceinline__ float4 router_rows_units(const T* xr0, const T* xr1, 
 // from zero and added to the total in fp32, so that its truncating accumulator
 // never carries a long sum (the gradient's error against 64 bits is 1.4e-7 at 2048 rows
 // of 2048 features, 7.9e-7 as serial fp32 sums).
-// Returns what router_rows_units returns; smem: RED_FLOATS floats.
 __device__ __forceinline__ void mma_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
                                           uint32_t b1) {
   asm volatile(
@@ -162,7 +161,8 @@ struct RouterPiece {
   }
 };
 // The sums over pieces [c_lo, c_hi), which the warps take in turn; `next` holds the
-// weights of the warp's first piece (c_lo + warp) if there is one.
+// weights of the warp's first piece (c_lo + warp) if there is one. Returns what
+// router_rows_units returns; smem: RED_FLOATS floats.
 __device__ __forceinline__ float4 router_rows_partial(const bf16* xr0, const bf16* xr1, const bf16* w1, int d, int c_lo,
                                                       int c_hi, RouterPiece& next, float* smem) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
