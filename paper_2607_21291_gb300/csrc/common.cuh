@@ -305,8 +305,10 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
-// All threads of every CTA of the cluster.
+// All threads of every CTA of the cluster. The barriers are warp-aligned: the
+// warp rejoins first, whatever loop or branch its lanes come from.
 __device__ __forceinline__ void cluster_sync() {
+  __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
@@ -378,6 +380,7 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
 }
 // Barrier among `nthreads` threads (whole warps) on named barrier `id` (1..15).
 __device__ __forceinline__ void named_bar_sync(int id, int nthreads) {
+  __syncwarp();   // bar.sync is warp-aligned
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 // One warp in each CTA of the pair: allocate `ncols` TMEM columns in both.
