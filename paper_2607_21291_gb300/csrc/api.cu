@@ -55,9 +55,25 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 
 int elem_size(int dtype) { return dtype == kBF16 ? 2 : 4; }
 
+// A host thread that has not used CUDA yet has no current context, which a launch
+// would give it but the encoding of a tensor map refuses to do without.
+cudaError_t bind_context(int device) {
+  using GetCurrent = CUresult (*)(CUcontext*);
+  static const GetCurrent get = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    const cudaError_t e = cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &p, 12000, cudaEnableDefault, &q);
+    return e == cudaSuccess && q == cudaDriverEntryPointSuccess ? reinterpret_cast<GetCurrent>(p) : nullptr;
+  }();
+  CUcontext ctx = nullptr;
+  if (get && get(&ctx) == CUDA_SUCCESS && ctx) return cudaSuccess;
+  return cudaSetDevice(device);
+}
+
 adadsf_status device_info(Dev* dev, void* stream, void* ws) {
   int device = 0;
   CUDA_TRY(cudaGetDevice(&device), "cudaGetDevice");
+  CUDA_TRY(bind_context(device), "current context");
   static int sms[64] = {0};
   if (device >= 64) return fail(ADADSF_ERR_UNSUPPORTED, "device ordinal %d >= 64", device);
   if (!sms[device]) {

@@ -1,6 +1,9 @@
 """GPU parity of the individual steps against the fp64 oracle, through the C ABI.
 Sizes span several tiles with ragged tails; edge cases include K = 0, 1, T-1, T,
 ties, NaN and signed zeros."""
+import ctypes
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -188,6 +191,46 @@ def test_linear_bf16_few_rows_streamed(A, M, N, Kd, act):
     again = torch.empty_like(out[:M])
     A.adadsf_linear(x, w, b, again, act=act, ws=ws)
     assert torch.equal(again, out[:M])
+
+
+@pytest.mark.parametrize("entry", ["linear", "linear_few_rows", "router", "align_output"])
+def test_first_cuda_call_of_a_host_thread(A, entry):
+    """A thread's first use of CUDA is a call whose kernel loads through tensor
+    maps: it is accepted and gives what the main thread gets."""
+    g = torch.Generator(device="cuda").manual_seed(6)
+    rnd = lambda *shape: torch.randn(shape, generator=g, device="cuda").bfloat16()
+    p = lambda t: ctypes.c_void_p(t.data_ptr())
+    stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    if entry.startswith("linear"):
+        x, w = rnd(16 if entry == "linear_few_rows" else 300, 2048), rnd(4608, 2048)
+        out, ws = torch.empty(x.shape[0], 4608, dtype=torch.bfloat16, device="cuda"), A.workspace(256)
+        fn, keep = A.lib().adadsf_linear, (x, w)
+        args = (p(x), p(w), None, x.shape[0], 4608, 2048, A.DTYPE_CODE[x.dtype], 0, p(out), p(ws), ws.numel(), stream)
+    elif entry == "router":
+        shape = S.PYTHIA_160M.replace(n_layers=1)
+        w, x = A.to_device(H.host_layer(shape, 3), torch.bfloat16), rnd(8192, shape.d)
+        cfg, lw = A.make_cfg(shape), A.layer_struct(w)
+        out, ws = torch.empty(8192, device="cuda"), A.workspace(256)
+        fn, keep = A.lib().adadsf_router_scores, (x, w)
+        args = (ctypes.byref(cfg), ctypes.byref(lw), p(x), 8192, p(out), p(ws), ws.numel(), stream)
+    else:
+        hs, hd, head = rnd(200, 512), rnd(200, 512), rnd(640, 512)
+        out = torch.zeros(2, dtype=torch.float64, device="cuda")
+        ws = A.workspace(A.lib().adadsf_align_workspace_size(200, 640))
+        fn, keep = A.lib().adadsf_align_output, (hs, hd, head)
+        args = (p(hs), p(hd), p(head), 200, 512, 640, A.DTYPE_CODE[hs.dtype], p(out), p(ws), ws.numel(), stream)
+    torch.cuda.synchronize()
+    assert fn(*args) == A.OK
+    torch.cuda.synchronize()
+    ref = out.clone()
+    out.zero_()
+    torch.cuda.synchronize()
+    status = []
+    t = threading.Thread(target=lambda: status.append(fn(*args)))
+    t.start()
+    t.join()
+    torch.cuda.synchronize()
+    assert status == [A.OK] and torch.equal(out, ref) and len(keep)
 
 
 @pytest.mark.parametrize("M,N,Kd,act", [(1, 4, 4, 0), (63, 36, 100, 1), (65, 516, 2052, 0), (129, 68, 64, 1),
