@@ -203,7 +203,7 @@ cudaError_t launch_attn_f32(const float* q, int64_t ld_qkv, float* o, int64_t ld
                             int n_kv_heads, const Dev& dev) {
   const int64_t blocks = (int64_t)((K + kAtQ - 1) / kAtQ) * n_heads * B;
   if (blocks > INT32_MAX) return cudaErrorInvalidValue;
-  const cudaError_t e = allow_smem(attn_f32_kernel<HD>, AttnF32<HD>::SMEM);
+  const cudaError_t e = allow_smem<attn_f32_kernel<HD>, AttnF32<HD>::SMEM>();
   if (e != cudaSuccess) return e;
   return launch_pdl(attn_f32_kernel<HD>, dim3((unsigned)blocks), dim3(kAtThreads), AttnF32<HD>::SMEM, dev.stream, q,
                     ld_qkv, o, ld_out, K, n_heads, n_kv_heads, B, 1.f / sqrtf((float)HD));

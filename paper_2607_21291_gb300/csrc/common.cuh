@@ -7,6 +7,8 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "internal.h"
 
 namespace adadsf {
@@ -460,10 +462,24 @@ __device__ __forceinline__ void decide_row(int b, const float* scores, const flo
   if (kept_out) kept_out[b] = keep ? 1 : 0;
 }
 
-// Host: let `kernel` use `bytes` of dynamic shared memory on the current device.
-template <typename K>
-inline cudaError_t allow_smem(K kernel, int bytes) {
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+// Host: let KERNEL use up to BYTES of dynamic shared memory on the current device. The
+// limit belongs to the function and the device, not to a launch: a call that set
+// its own size could lower it between another host thread's call and that thread's
+// launch, which was then refused (8186 of 20,000 products of 4608 columns beside a
+// thread's products of 512). So it is one constant per kernel, the most any of its launches asks for,
+// set once per device.
+template <auto KERNEL, int BYTES>
+inline cudaError_t allow_smem() {
+  static_assert(BYTES <= 232448, "past what a block may ask for");
+  static std::atomic<bool> done[64];
+  int device = 0;
+  cudaError_t e = cudaGetDevice(&device);
+  if (e != cudaSuccess) return e;
+  const bool known = device >= 0 && device < 64;
+  if (known && done[device].load(std::memory_order_acquire)) return cudaSuccess;
+  e = cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, BYTES);
+  if (e == cudaSuccess && known) done[device].store(true, std::memory_order_release);
+  return e;
 }
 
 // Host: launch `kernel` on `stream` with programmatic stream serialisation.

@@ -640,7 +640,7 @@ cudaError_t cache_header(int32_t* hdr, int T, int C_max, int L, int B, const Dev
 template <int HD, bool CLUSTER>
 static cudaError_t launch_decode_tc(const CUtensorMap& tk, const CUtensorMap& tv, const DecodeAttn& a, int ns,
                                     float scale_log2, const Dev& dev) {
-  const cudaError_t e = allow_smem(decode_attn_tc_kernel<HD, CLUSTER>, DecTc<HD>::SMEM);
+  const cudaError_t e = allow_smem<decode_attn_tc_kernel<HD, CLUSTER>, DecTc<HD>::SMEM>();
   if (e != cudaSuccess) return e;
   const dim3 grid(ns, a.Hkv, a.B);
   const bf16* q = static_cast<const bf16*>(a.qkv);

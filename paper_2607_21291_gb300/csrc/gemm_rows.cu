@@ -223,6 +223,10 @@ constexpr int kGsGroups = 8;          // 8-row groups of W a tile takes
 constexpr int kGsBox = 2048;          // bytes of 8 rows x 128 k
 constexpr int kGsMaxStages = 12;
 constexpr int kGsRingBytes = 184 * 1024;
+// Shared memory of a launch: alignment, the ring, the warps' sums and the peer's half.
+constexpr int gs_smem(int ring, int pairs, int nt) {
+  return 1024 + ring + (kGsWarps * pairs * 16 + pairs * 8) * nt * 8 * 4;
+}
 
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const void* tmap, int c0, int c1, int c2, uint32_t bar) {
   asm volatile(
@@ -477,8 +481,8 @@ cudaError_t launch_stream(const GemmArgs& a, const RowsDev& p, const Dev& dev) {
   if (a.K2 > 0 && (!map(&w2, a.Wk2, a.N, a.K2, a.ldwk2, 8 * U) || !map(&x2, a.A2, a.M, a.K2, a.lda2, 8 * NT)))
     return cudaErrorInvalidValue;
   const int stage = (U + NT) * kGsBox, S = std::min(kGsMaxStages, kGsRingBytes / stage);
-  const int smem = 1024 + S * stage + (kGsWarps * pairs * 16 + pairs * 8) * NT * 8 * 4;
-  const cudaError_t e = allow_smem(gemm_rows_stream_kernel<NT>, smem);
+  const int smem = gs_smem(S * stage, pairs, NT);
+  const cudaError_t e = allow_smem<gemm_rows_stream_kernel<NT>, gs_smem(kGsRingBytes, kGsGroups / 2, NT)>();
   if (e != cudaSuccess) return e;
   return launch_pdl(gemm_rows_stream_kernel<NT>, dim3((unsigned)(2 * ncl)), dim3(kGsThreads), (size_t)smem, dev.stream, w,
                     x, w2, x2, p, U, S, dev.err, kWaitTimeoutNs);

@@ -309,7 +309,7 @@ cudaError_t launch_f32(const SimtDev& a, const SimtDev& b, int S, const Dev& dev
   auto tiles = [](const SimtDev& p) { return (((int64_t)p.M + BM - 1) / BM) * ((p.N + NOUT - 1) / NOUT); };
   const int64_t ctas = (tiles(a) + tiles(b)) * S;
   if (ctas > INT32_MAX) return cudaErrorInvalidValue;
-  cudaError_t e = allow_smem(gemm_f32_kernel<BM, BN, TM, TN, KS, DUAL>, C::SMEM);
+  const cudaError_t e = allow_smem<gemm_f32_kernel<BM, BN, TM, TN, KS, DUAL>, C::SMEM>();
   if (e != cudaSuccess) return e;
   if (S == 1)
     return launch_pdl(gemm_f32_kernel<BM, BN, TM, TN, KS, DUAL>, dim3((unsigned)ctas), dim3(C::THREADS), C::SMEM,

@@ -330,7 +330,7 @@ cudaError_t kl_tc(const void* hs, const void* hd, const void* w, int64_t n_rows,
                   double* partials, double* acc, const Dev& dev) {
   if (n_rows <= 0) return cudaSuccess;
   if (n_rows > INT32_MAX - kKlM || n_cls % 64 || d % 64) return cudaErrorInvalidValue;
-  cudaError_t e = allow_smem(kl_tc_kernel, kKlSmem);
+  cudaError_t e = allow_smem<kl_tc_kernel, kKlSmem>();
   if (e != cudaSuccess) return e;
   CUtensorMap ts, td, tw;
   if (!make_tmap_bf16(&ts, hs, (uint64_t)n_rows, (uint64_t)d, (uint64_t)d, kKlK, kKlM) ||

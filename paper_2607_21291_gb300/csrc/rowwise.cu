@@ -966,13 +966,16 @@ cudaError_t decide_norm(int dtype, const void* x, int B, int d, bool is_rms, con
 
 bool decode_front_fits(int dtype, int B, int h) { return dtype == kBF16 && B <= kFrontRows && h == kRrUnits; }
 
+// Shared memory of a launch: the warps' partial tiles, this CTA's share and the norm parameters.
+constexpr int front_smem(int d) { return (RouterRows<bf16>::RED_FLOATS + kRrRows * kRrUnits) * 4 + 4 * d * 2; }
+
 template <bool RMS>
 cudaError_t decode_front_t(const DecodeFront& a, const Dev& dev) {
   auto p = [](const void* v) { return static_cast<const bf16*>(v); };
-  const int smem = (RouterRows<bf16>::RED_FLOATS + kRrRows * kRrUnits) * 4 + 4 * a.d * 2;
+  const int smem = front_smem(a.d);
   return with_nch<bf16>(a.d, [&](auto nch) -> cudaError_t {
     constexpr int NCH = decltype(nch)::value;
-    const cudaError_t e = allow_smem(decode_front_kernel<RMS, NCH>, smem);
+    const cudaError_t e = allow_smem<decode_front_kernel<RMS, NCH>, front_smem(NCH * 32 * Elem<bf16>::kVec)>();
     if (e != cudaSuccess) return e;
     return launch_pdl_cluster(decode_front_kernel<RMS, NCH>, dim3(kFrontCluster), dim3(kRrThreads), (size_t)smem,
                               dev.stream, kFrontCluster, p(a.x), a.B, a.d, p(a.w1), p(a.rb1), p(a.w2), p(a.rb2), p(a.g1),
@@ -1026,7 +1029,7 @@ cudaError_t rope_apply(int dtype, void* qkv, int64_t M, int64_t ld, int n_heads,
 cudaError_t router_f32(const float* x, int64_t n, int d, int h, const float* w1, const float* b1,
                        const float* w2, const float* b2, float* scores, const Dev& dev) {
   if (n <= 0) return cudaSuccess;
-  const cudaError_t e = allow_smem(router_f32_kernel, RouterRows<float>::SMEM_BYTES);
+  const cudaError_t e = allow_smem<router_f32_kernel, RouterRows<float>::SMEM_BYTES>();
   if (e != cudaSuccess) return e;
   return launch_pdl(router_f32_kernel, dim3((unsigned)((n + kRrRows - 1) / kRrRows)), dim3(kRrThreads),
                     RouterRows<float>::SMEM_BYTES, dev.stream, x, n, d, h, w1, b1, w2, b2, scores);
@@ -1107,7 +1110,7 @@ cudaError_t router_rows16(const void* x, int64_t n_rows, int d, const void* w1, 
   int C = 8;
   while (C > 1 && tiles * C > 2 * dev.num_sms) C /= 2;
   constexpr int smem = (RouterRows<bf16>::RED_FLOATS + kRrRows * kRrUnits) * 4;
-  const cudaError_t e = allow_smem(router_rows16_kernel, smem);
+  const cudaError_t e = allow_smem<router_rows16_kernel, smem>();
   if (e != cudaSuccess) return e;
   return launch_pdl_cluster(router_rows16_kernel, dim3((unsigned)(tiles * C)), dim3(kRrThreads), (size_t)smem, dev.stream,
                             C, static_cast<const bf16*>(x), n_rows, d, static_cast<const bf16*>(w1),

@@ -593,7 +593,7 @@ cudaError_t router_backward_t(const void* x, const void* y_plain, const int32_t*
   const int64_t nb = (M + kRrRows - 1) / kRrRows;
   if (nb > INT32_MAX) return cudaErrorInvalidValue;
   constexpr int smem = sizeof(T) == 2 ? RouterRows<T>::MMA_BYTES : RouterRows<T>::SMEM_BYTES;
-  cudaError_t e = allow_smem(router_bwd_rows_kernel<T>, smem);
+  cudaError_t e = allow_smem<router_bwd_rows_kernel<T>, smem>();
   if (e != cudaSuccess) return e;
   const int vec = (reinterpret_cast<uintptr_t>(G) & 15u) == 0 ? 1 : 0;
   e = launch_pdl(router_bwd_rows_kernel<T>, dim3((unsigned)nb), dim3(kRrThreads), smem, dev.stream,

@@ -233,6 +233,48 @@ def test_first_cuda_call_of_a_host_thread(A, entry):
     assert status == [A.OK] and torch.equal(out, ref) and len(keep)
 
 
+def test_linear_from_two_host_threads(A):
+    """Streamed products of different column counts (so different sizes of the
+    same kernel's ring) enqueued by two host threads on streams of their own:
+    none is refused, and each output is the one it gets alone. The calls go
+    straight to the library, whose part of a call outside the interpreter's lock
+    is then the longer one: the threads meet there."""
+    g = torch.Generator(device="cuda").manual_seed(5)
+    rnd = lambda *shape: torch.randn(shape, generator=g, device="cuda").bfloat16()
+    jobs = [(rnd(16, k), rnd(n, k)) for n, k in ((4608, 2048), (512, 20480))]
+    outs = [torch.empty(16, w.shape[0], dtype=torch.bfloat16, device="cuda") for _, w in jobs]
+    wss, streams = [A.workspace(256) for _ in jobs], [torch.cuda.Stream() for _ in jobs]
+    fn = A.lib().adadsf_linear
+    vp = ctypes.c_void_p
+    calls = [(vp(x.data_ptr()), vp(w.data_ptr()), None, 16, w.shape[0], w.shape[1], A.DTYPE_CODE[x.dtype], 0,
+              vp(o.data_ptr()), vp(ws.data_ptr()), ws.numel(), vp(st.cuda_stream))
+             for (x, w), o, ws, st in zip(jobs, outs, wss, streams)]
+    torch.cuda.synchronize()
+    assert [fn(*c) for c in calls] == [A.OK, A.OK]
+    torch.cuda.synchronize()
+    alone = [o.clone() for o in outs]
+    for o in outs:
+        o.zero_()
+    torch.cuda.synchronize()
+    refused, last, start = [0, 0], [], threading.Barrier(2)
+
+    def work(i):
+        start.wait()
+        for _ in range(20000):
+            if fn(*calls[i]) != A.OK:
+                refused[i] += 1
+                last.append(A.adadsf_last_error())
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert refused == [0, 0], last
+    assert all(A.adadsf_sync_check(ws) == A.OK for ws in wss)
+    assert torch.equal(outs[0], alone[0]) and torch.equal(outs[1], alone[1])
+
+
 @pytest.mark.parametrize("M,N,Kd,act", [(1, 4, 4, 0), (63, 36, 100, 1), (65, 516, 2052, 0), (129, 68, 64, 1),
                                         (64, 512, 2048, 0), (700, 2048, 96, 1), (1532, 512, 2048, 0), (3001, 260, 36, 1)])
 def test_linear_f32_splits(A, M, N, Kd, act):

@@ -7,6 +7,8 @@ sparse forward), and so are its per-step keep decisions; each decision must
 equal the oracle's own wherever the oracle's score is more than 1e-3 away
 from its threshold. Hidden states within the parity tolerance; cached counts
 follow the decisions; the cache's thresholds match the oracle's."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -307,3 +309,39 @@ def test_decode_on_two_streams_interleaved(A):
     assert A.adadsf_sync_check(wss[0]) == A.OK and A.adadsf_sync_check(wss[1]) == A.OK
     assert torch.equal(torch.stack(outs[0]), alone1)
     assert torch.equal(torch.stack(outs[1]), alone2)
+
+
+def test_decode_from_two_host_threads(A):
+    """Two host threads, each with a model, a cache and a stream of its own,
+    enqueue decode steps at the same time: models of different widths whose
+    launches are the same kernels at different shared-memory sizes (the norm
+    parameters of the first launch, the ring of the streamed projections). Each
+    gets the outputs it gets alone, and no step is refused. (24 layers that share
+    their weights: the library's part of a step is then longer than the
+    interpreter's, and the threads meet there.)"""
+    shapes = [NEOX_WIDE, NEOX_WIDE.replace(d=1792, n_heads=14, n_kv_heads=14, ffn=7168)]
+    B, T0, L, steps, C_max = 2, 24, 24, 60, 96
+    K = [20] * L
+    models = []
+    for i, s in enumerate(shapes):
+        one = _small_model(A, s, 81 + i)[0]
+        models.append(A.DeviceModel(A.make_cfg(s.replace(n_layers=L)), one.layers * L, one.extra))
+    ids = [torch.from_numpy(S.token_ids(83 + i, B, T0 + steps, s.vocab)).cuda() for i, s in enumerate(shapes)]
+    alone = [_decode_run(A, m, torch.bfloat16, t, B, T0, K, C_max, steps, torch.cuda.Stream())
+             for m, t in zip(models, ids)]
+    got, errors = [None, None], []
+    start = threading.Barrier(2)
+
+    def work(i):
+        try:
+            start.wait()
+            got[i] = _decode_run(A, models[i], torch.bfloat16, ids[i], B, T0, K, C_max, steps, torch.cuda.Stream())
+        except Exception as e:
+            errors.append(e)
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    assert torch.equal(got[0], alone[0]) and torch.equal(got[1], alone[1])
