@@ -15,7 +15,8 @@
  *    stream). Every device entry point only enqueues work on that stream
  *    (adadsf_decode_step may use a stream of its own that it joins back into
  *    it) and returns without synchronising; results are ready once the
- *    stream is.
+ *    stream is. Every operand, weights included, may be the output of work
+ *    enqueued on the stream before the call.
  *  - Tensors are dense row-major. Weights are [out_features, in_features]
  *    (the torch.nn.Linear layout); the fused QKV weight stacks the query
  *    rows, then the key rows, then the value rows.

@@ -153,7 +153,7 @@ struct Profiler {
 };
 Profiler g_prof;
 
-// Runs f() (which enqueues one kernel or copy on dev.stream); while profiling
+// Runs f() (which enqueues a kernel or copy on dev.stream); while profiling
 // is on and the stream is not being captured, brackets it with events.
 template <typename F>
 adadsf_status launch(const Dev& dev, int kind, bool dense, double flops, double bytes, F&& f) {
@@ -175,6 +175,7 @@ adadsf_status launch(const Dev& dev, int kind, bool dense, double flops, double 
   }
   const cudaError_t ea = a ? cudaEventRecord(a, dev.stream) : cudaSuccess;
   const adadsf_status st = f();
+  dev.behind_own = true;
   const cudaError_t eb = b ? cudaEventRecord(b, dev.stream) : cudaSuccess;
   if (ea != cudaSuccess || eb != cudaSuccess) {
     std::lock_guard<std::mutex> lk(g_prof.mu);

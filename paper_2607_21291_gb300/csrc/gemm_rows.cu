@@ -6,8 +6,8 @@
 // 128 weight rows, partial tiles exchanged between the CTAs of a split): a few MB of
 // weights took 8 to 15 us. Here a block takes 8-row groups of W, as evenly as the
 // groups divide, its 16 warps every sixteenth 64-byte piece of K, and the first pieces
-// are on their way before the block waits for the previous kernel (weights do not
-// depend on it). The product is warp-level (mma.sync m16n8k16): 16 weight rows
+// are on their way before the block waits for the previous kernel (which is one of
+// the same call, so that weights do not depend on it). The product is warp-level (mma.sync m16n8k16): 16 weight rows
 // are the A operand, the rows of A the B operand's columns. Both come straight from
 // memory: a lane loads 16 consecutive bytes of a row, and since the order of k inside
 // a product is free as long as both operands agree, those bytes are the fragment as
@@ -48,6 +48,7 @@ struct RowsDev {
   const bf16* x2; int64_t ldx2;       // second K source, pieces n1 ...
   const bf16* wk2; int64_t ldwk2;
   int M, groups, n1, n;               // groups: N / 8; pieces of 32 k: first source, both
+  int wait_first;                     // the weights may be the previous kernel's output
   int act;
   const bf16 *bias, *bias2;
   const bf16* add; int64_t ld_add; int add_gathered;   // residual
@@ -145,6 +146,7 @@ __global__ void __launch_bounds__(kGrThreads, 1)
       }
     }
   };
+  if (pa.wait_first) pdl_wait();
   Tile cur = {};
   if (lo < hi) {
     cur = tile_at(lo);
@@ -314,7 +316,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGsThreads, 1)
         const bool s2 = k >= n1;
         tma_load_3d(ring + s * stage_bytes + U * kGsBox, s2 ? &tmX2 : &tmX, 0, 0, 2 * (s2 ? k - n1 : k), full0 + 8 * s);
       };
-      // the weights of the first stages do not depend on the kernel before
+      // behind a launch of the same call the weights do not depend on the kernel before
+      if (p.wait_first) pdl_wait();
       const int pre = min(S, k1 - k0);
       for (int i = 0; i < pre; ++i) load_w(k0 + i, i);
       pdl_wait();
@@ -500,6 +503,7 @@ bool gemm_rows_takes(const GemmArgs& a, const GemmArgs* b, int num_sms) {
 cudaError_t gemm_rows(const GemmArgs& a, const GemmArgs* b, const Dev& dev) {
   RowsDev p, q = {};
   if (!rows_dev(a, p) || (b && !rows_dev(*b, q))) return cudaErrorInvalidValue;
+  p.wait_first = dev.behind_own ? 0 : 1;
   if (!b && streams(a, dev.num_sms)) return a.M <= 8 ? launch_stream<1>(a, p, dev) : launch_stream<2>(a, p, dev);
   const dim3 grid((unsigned)std::min(dev.num_sms, p.groups + q.groups)), block(kGrThreads);
   if (a.epi.act == ACT_SWIGLU)

@@ -115,6 +115,7 @@ struct GemmDev {
   float* sq_out; int sq_ld;
   float4* cos_out; int cos_ld;
   const bf16* cin; int64_t ld_cin;
+  int wait_first;            // the weights may be the previous kernel's output
   int* err;
   unsigned long long timeout_ns;
 };
@@ -738,8 +739,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       int64_t issued = 0;
       // bytes per stage: the A tile and this problem's weight tile(s)
       auto stage_tx = [&](int bn) { return (uint32_t)(p.a_box_rows * BK * 2 + bn * BK * 2 * C::NUM_B); };
-      // The weights do not depend on the previous kernel: the first tile's
-      // weight tiles are requested before waiting for it.
+      // Behind a launch of the same call the weights do not depend on the previous
+      // kernel: the first tile's weight tiles are requested before waiting for it.
+      if (p.wait_first) pdl_wait();
       int pre = 0;
       if ((int)blockIdx.x < num_tiles) {
         const TileInfo ti = tile_info(blockIdx.x, p, p2, tiles0, BM);
@@ -959,6 +961,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (lane == 0) {
       const uint32_t tx = (uint32_t)(p.a_box_rows * BK * 2 + C::B_BYTES);
       const int npre = nkb < C::STAGES ? nkb : C::STAGES;
+      if (p.wait_first) pdl_wait();
       for (int i = 0; i < npre; ++i) {   // weights first: independent of the previous kernel
         const KbSrc src = kb_source(ti, kb0 + i, &tmA, &tmB, &tmA2, &tmB2);
         mbar_arrive_expect_tx(full0 + 8 * i, tx);
@@ -1160,6 +1163,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     uint32_t phase = 0;
     int64_t issued = 0;
     constexpr uint32_t tx = 2 * C::STAGE_BYTES;
+    if (p.wait_first) pdl_wait();
     int pre = 0;
     if (pair < num_tiles) {
       const TileInfo ti = tile_info(pair, p, p2, tiles0, 2 * BM);
@@ -1221,6 +1225,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       // both CTAs' bytes; the odd CTA's copies complete transactions on it,
       // possibly before it is armed (the transaction count may go negative).
       constexpr uint32_t tx = 2 * C::STAGE_BYTES;
+      if (p.wait_first) pdl_wait();
       int pre = 0;
       if (pair < num_tiles) {
         const TileInfo ti = tile_info(pair, p, p2, tiles0, 2 * BM);
@@ -1463,6 +1468,7 @@ bool make_dev(const GemmArgs& a, const Dev& dev, GemmDev& p) {
   p.vt_hkv = a.epi.vt_hkv;
   p.scratch = a.scratch;
   p.err = dev.err;
+  p.wait_first = dev.behind_own ? 0 : 1;
   p.timeout_ns = kWaitTimeoutNs;
   return true;
 }

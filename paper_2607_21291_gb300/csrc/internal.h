@@ -113,6 +113,11 @@ struct Dev {
   cudaStream_t stream;
   int* err;          // device error word
   int num_sms;
+  // Whether an earlier launch of the same call precedes on the stream. Such a launch
+  // has waited for whatever the caller enqueued before, so the kernels behind it may
+  // read weights before their own pdl_wait(). The first one may not: the kernel
+  // before it can be the one that writes them.
+  mutable bool behind_own = false;
 };
 
 // Tensor map of a row-major bf16 [rows, cols] matrix (leading dimension ld

@@ -79,6 +79,7 @@ struct RouterDev {
   float* tsq;            // [rows] sum of squares of each token row of X, or null
   float* partials;       // [G][2][kRSlot]
   int* tile_cnt;         // [G]: split tile counted at its first CTA
+  int wait_first;        // W1 and the rest may be the previous kernel's output
   int* err;
   unsigned long long timeout_ns;
 };
@@ -155,8 +156,9 @@ __global__ void __launch_bounds__(kRThreads, 1)
     if (lane == 0) {
       const int64_t n = u1 - u0;
       const int pre = (int)(n < kRStages ? n : kRStages);
-      // W1 does not depend on the previous kernel: the first stages' weight
-      // tiles are requested before waiting for it
+      // behind a launch of the same call W1 does not depend on the previous kernel:
+      // the first stages' weight tiles are requested before waiting for it
+      if (p.wait_first) pdl_wait();
       for (int i = 0; i < pre; ++i) {
         const int kb = (int)((u0 + i) % p.nkb);
         mbar_arrive_expect_tx(full0 + 8 * i, kRA + kRB);
@@ -235,7 +237,8 @@ __global__ void __launch_bounds__(kRThreads, 1)
     const int r = quarter * 32 + lane;      // token in the tile
     const int etid = threadIdx.x - 64;
     const auto esync = [] { named_bar_sync(kRBar, kREpiThreads); };
-    if (etid < kRN) {   // weights: independent of the previous kernel
+    if (p.wait_first) pdl_wait();
+    if (etid < kRN) {   // weights: as above
       cst[etid] = __bfloat162float(p.b1[etid]);
       cst[kRN + etid] = __bfloat162float(p.w2[etid]);
     }
@@ -496,6 +499,7 @@ cudaError_t router_tc(const void* x, int64_t rows, int d, const void* w1, const 
   p.tsq = tsq;
   p.tile_cnt = sync;
   p.partials = partials;
+  p.wait_first = dev.behind_own ? 0 : 1;
   p.err = dev.err;
   p.timeout_ns = kWaitTimeoutNs;
   CUtensorMap tx, tw;

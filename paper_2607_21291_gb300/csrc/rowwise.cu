@@ -179,16 +179,18 @@ __device__ __forceinline__ void norm_share(int64_t lo, int64_t hi, const T* x, i
 // ---------------------------------------------------------------- few rows
 // Gather + norm of a few rows (a decode step's one row per sequence): four
 // warps per block, one row per warp, the row in registers; the parameters
-// are staged before waiting for the previous kernel (they do not depend on it).
+// are staged before waiting for the previous kernel (they do not depend on one of
+// the same call; wait_first: it is the caller's).
 constexpr int kFewRowWarps = 4;
 constexpr int64_t kFewRowsMax = 512;   // larger counts stream through gather_norm_tma_kernel
 
 template <typename T, bool RMS, int NCH>
 __global__ void __launch_bounds__(32 * kFewRowWarps)
     norm_few_rows_kernel(const T* x, const int32_t* rows, int64_t M, int d, const T* g1, const T* b1,
-                         const T* g2, const T* b2, float eps, T* out1, T* out2) {
+                         const T* g2, const T* b2, float eps, T* out1, T* out2, int wait_first) {
   extern __shared__ __align__(16) uint8_t smem_few[];
   T* sp = reinterpret_cast<T*>(smem_few);
+  if (wait_first) pdl_wait();
   stage_norm_params(g1, RMS ? nullptr : b1, out2 ? g2 : nullptr, (RMS || !out2) ? nullptr : b2, d, sp);
   pdl_wait();
   pdl_trigger();
@@ -306,7 +308,7 @@ __global__ void __launch_bounds__(kRrThreads)
 // Error against 64 bits 1.2e-7 (5.6e-7 to 1.9e-6 there).
 __global__ void __launch_bounds__(kRrThreads)
     router_rows16_kernel(const bf16* x, int64_t n_rows, int d, const bf16* w1, const bf16* rb1, const bf16* w2,
-                         const bf16* rb2, float* scores) {
+                         const bf16* rb2, float* scores, int wait_first) {
   extern __shared__ __align__(16) uint8_t smem_r16[];
   float* red = reinterpret_cast<float*>(smem_r16);                       // [warp][16][64]
   float* part = red + RouterRows<bf16>::RED_FLOATS;                     // [16][64]: this CTA's share
@@ -315,8 +317,9 @@ __global__ void __launch_bounds__(kRrThreads)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n = d / 32;                                                 // pieces of 32 features
   const int c_lo = n * rank / C, c_hi = n * (rank + 1) / C;
+  if (wait_first) pdl_wait();
   RouterPiece pc;
-  if (c_lo + warp < c_hi) pc.load_w(w1, d, c_lo + warp);                // weights: independent of the previous kernel
+  if (c_lo + warp < c_hi) pc.load_w(w1, d, c_lo + warp);                // weights: independent of a launch of the same call
   pdl_wait();
   pdl_trigger();
   const int64_t ra = min(r0 + (lane >> 2), n_rows - 1), rb = min(r0 + 8 + (lane >> 2), n_rows - 1);
@@ -388,7 +391,7 @@ template <typename T, bool RMS, int NCH>
 __global__ void __launch_bounds__(kRowThreads)
     gather_norm_tma_kernel(const T* x, const int32_t* rows, int64_t M, int d, const T* g1,
                            const T* b1, const T* g2, const T* b2, float eps, T* out1, T* out2,
-                           int* err, unsigned long long timeout_ns) {
+                           int* err, unsigned long long timeout_ns, int wait_first) {
   extern __shared__ __align__(16) uint8_t smem_rows[];
   constexpr int V = Elem<T>::kVec;
   const uint32_t row_bytes = (uint32_t)d * sizeof(T);
@@ -406,8 +409,9 @@ __global__ void __launch_bounds__(kRowThreads)
     abort_flag = 0;
     fence_barrier_init();
   }
+  if (wait_first) pdl_wait();
   stage_norm_params(g1, RMS ? nullptr : b1, out2 ? g2 : nullptr, (RMS || !out2) ? nullptr : b2, d,
-                    sp);   // weights: independent of the previous kernel (also syncs the block)
+                    sp);   // weights: independent of a previous kernel of the same call (also syncs the block)
   pdl_wait();
   pdl_trigger();
   const int64_t lo = (int64_t)blockIdx.x * M / gridDim.x, hi = (int64_t)(blockIdx.x + 1) * M / gridDim.x;
@@ -915,7 +919,7 @@ cudaError_t gather_norm_launch(const void* x, const int32_t* rows, int64_t M, in
                     dev.stream, static_cast<const T*>(x), rows, M, d, static_cast<const T*>(g1),
                     static_cast<const T*>(b1), static_cast<const T*>(g2),
                     static_cast<const T*>(b2), eps, static_cast<T*>(out1), static_cast<T*>(out2),
-                    dev.err, kWaitTimeoutNs);
+                    dev.err, kWaitTimeoutNs, dev.behind_own ? 0 : 1);
 }
 
 template <typename T, bool RMS>
@@ -928,7 +932,8 @@ cudaError_t gather_norm_t(const void* x, const int32_t* rows, int64_t M, int d, 
       return launch_pdl(norm_few_rows_kernel<T, RMS, NCH>, dim3((unsigned)((M + kFewRowWarps - 1) / kFewRowWarps)),
                         dim3(32 * kFewRowWarps), 4 * (size_t)d * sizeof(T), dev.stream, static_cast<const T*>(x), rows,
                         M, d, static_cast<const T*>(g1), static_cast<const T*>(b1), static_cast<const T*>(g2),
-                        static_cast<const T*>(b2), eps, static_cast<T*>(out1), static_cast<T*>(out2));
+                        static_cast<const T*>(b2), eps, static_cast<T*>(out1), static_cast<T*>(out2),
+                        dev.behind_own ? 0 : 1);
     return gather_norm_launch<T, RMS, NCH>(x, rows, M, d, g1, b1, g2, b2, eps, out1, out2, dev);
   });
 }
@@ -1115,7 +1120,7 @@ cudaError_t router_rows16(const void* x, int64_t n_rows, int d, const void* w1, 
   return launch_pdl_cluster(router_rows16_kernel, dim3((unsigned)(tiles * C)), dim3(kRrThreads), (size_t)smem, dev.stream,
                             C, static_cast<const bf16*>(x), n_rows, d, static_cast<const bf16*>(w1),
                             static_cast<const bf16*>(b1), static_cast<const bf16*>(w2), static_cast<const bf16*>(b2),
-                            scores);
+                            scores, dev.behind_own ? 0 : 1);
 }
 
 // Fixed block count for a given row count (independent of the device), so the

@@ -520,3 +520,75 @@ def test_layer_stats_row_groups(A, n, d, dtype):
     assert acc[1].item() == n
     assert acc[0].item() == pytest.approx((dot / (na.sqrt() * nb.sqrt())).sum().item(), rel=1e-5)
     assert flat.tolist() == pytest.approx([dot.sum().item(), na.sum().item(), nb.sum().item()], rel=1e-5)
+
+
+# ---------------------------------------------------------------- weights written just before
+@pytest.mark.parametrize("M,N,Kd", [(3, 768, 1024), (8, 1024, 14336), (16, 4608, 2048), (60, 1024, 2048), (300, 512, 1024),
+                                    (4096, 1024, 2048)])
+def test_linear_on_weights_written_just_before(A, M, N, Kd):
+    """A product whose weights the call before it on the stream writes (every
+    kernel that requests weights ahead of its turn: direct and streamed few-row
+    products, split along K, one and two CTAs a tile): the weights are the new
+    ones, to the bit what the product gives after a synchronisation."""
+    g = torch.Generator(device="cuda").manual_seed(M + N)
+    rnd = lambda *shape: torch.randn(shape, generator=g, device="cuda").bfloat16()
+    x, mix = rnd(M, Kd), (rnd(Kd, 512) / 16).bfloat16()
+    base = [rnd(N, 512) for _ in range(6)]
+    w, out = torch.zeros(N, Kd, dtype=torch.bfloat16, device="cuda"), rnd(M, N)
+    ws = A.workspace(A.LINEAR_SPLIT_WS_BYTES)
+    got = []
+    for b in base:
+        A.adadsf_linear(b, mix, None, w, ws=ws)
+        A.adadsf_linear(x, w, None, out, ws=ws)
+        got.append(out.clone())
+    assert A.adadsf_sync_check(ws) == A.OK
+    for b, o in zip(base, got):
+        A.adadsf_linear(b, mix, None, w, ws=ws)
+        torch.cuda.synchronize()
+        A.adadsf_linear(x, w, None, out, ws=ws)
+        assert torch.equal(out, o)
+
+
+@pytest.mark.parametrize("n", [100, 2000, 8192])
+def test_router_on_weights_written_just_before(A, n):
+    """The same for router scores whose W1 (and the rest) was just written."""
+    shape = S.PYTHIA_160M.replace(n_layers=1, d=2048)
+    W = [A.to_device(H.host_layer(shape, 5 + i), torch.bfloat16) for i in range(2)]
+    x = H.to_dev(S.hidden(n, 1, n, shape.d)[0], torch.bfloat16)
+    g = torch.Generator(device="cuda").manual_seed(n)
+    mix = (torch.randn((shape.d, shape.d), generator=g, device="cuda") / 32).bfloat16()
+    live = {k: v.clone() for k, v in W[0].items()}
+    cfg, ws = A.make_cfg(shape), A.workspace(256)
+    sc = torch.empty(n, device="cuda")
+
+    def scores(src, wait):
+        A.adadsf_linear(src["router_w1"], mix, None, live["router_w1"], ws=ws)
+        if wait:
+            torch.cuda.synchronize()
+        A.adadsf_router_scores(cfg, live, x, sc)
+        return sc.clone()
+    got = [scores(W[i % 2], False) for i in range(6)]
+    ref = [scores(W[i], True) for i in range(2)]
+    assert all(torch.equal(s, ref[i % 2]) for i, s in enumerate(got)) and not torch.equal(*ref)
+
+
+@pytest.mark.parametrize("rot", [0, 64])
+def test_layer_on_weights_folded_just_before(A, rot):
+    """A dense layer right behind adadsf_fold_norms of its weights; without
+    rotary its norm is the first launch, which reads what the folding stores last."""
+    shape = S.PYTHIA_160M.replace(n_layers=1, rotary_dim=rot)
+    cfg = A.make_cfg(shape)
+    x0 = H.to_dev(S.hidden(9, 2, 64, shape.d), torch.bfloat16)
+    ws = A.workspace(A.adadsf_layer_workspace_size(cfg, 2, 64, 64))
+    outs = []
+    for wait in (False, False, True):
+        W = A.to_device(H.host_layer(shape, 6), torch.bfloat16)
+        x = x0.clone()
+        torch.cuda.synchronize()
+        A.adadsf_fold_norms(cfg, W)
+        if wait:
+            torch.cuda.synchronize()
+        A.adadsf_sparse_layer_forward(cfg, W, x, 64, ws=ws)
+        outs.append(x)
+    assert A.adadsf_sync_check(ws) == A.OK
+    assert torch.equal(outs[0], outs[2]) and torch.equal(outs[1], outs[2])
