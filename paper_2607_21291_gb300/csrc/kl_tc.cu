@@ -5,7 +5,7 @@
 // TMEM accumulators (tcgen05.mma, M = N = 128, fp32), and its epilogue folds the
 // tile into running sums per row:
 //   Zs = sum e^(ls - ms),  Zd = sum e^(ld - md),  X = sum e^(ld - md) (ld - ls)
-// (ms, md near the running maxima), from which KL = X / Zd + log(Zs / Zd) + ms - md.
+// (ms, md the running maxima), from which KL = X / Zd + log(Zs / Zd) + ms - md.
 // Storing the logits and reading them back cost more than the products: 4 bytes
 // written and three times read per class, row and model (2 GB at 1000 rows of
 // 50304 classes). There the whole loss took 1492 us (two projections of 123 us
@@ -14,9 +14,10 @@
 // from HBM once, since the row blocks walk the classes side by side.
 //
 // Tiles are numbered row block major and the persistent CTAs take equal
-// contiguous ranges, so a CTA stays on one row block (two at most, with as many
-// tiles as CTAs) and keeps its sums in registers: one thread per row and half of
-// a tile's columns. At the end of a row block's tiles it writes the five sums;
+// contiguous ranges, so a CTA stays on one row block (parts of two, or with few
+// classes and many rows several whole ones) and keeps its sums in registers: one
+// thread per row and half of a tile's columns. At the end of a row block's tiles it
+// writes the five sums;
 // kl_merge_kernel adds each row's records in a fixed order, in double.
 //   warp 0     TMA: hs, hd and W tiles of 64 k, 4 stages of 48 KB
 //   warp 1     TMEM, MMA issue (one thread); accumulators double-buffered
@@ -56,9 +57,9 @@ __host__ __device__ __forceinline__ int kl_owner(int64_t tiles, int G, int64_t t
   return (int)(((t + 1) * G - 1) / tiles);
 }
 
-// Running sums of a row in units of 2^(l log2(e) - M): M the rounded running
-// maximum in those units (any M near the maximum serves; the records carry
-// the M that was used, so its rounding drops out).
+// Running sums of a row; ms, md: its running maxima, which differences are taken
+// from before they are scaled to powers of two (scaled maxima would leave their own
+// rounding in the exponent, past any bound from logits near 1e9 on).
 struct KlSums {
   float ms, zs, md, zd, x;
 };
@@ -80,17 +81,18 @@ __device__ __forceinline__ void kl_fold(KlSums& s, const uint32_t* us, const uin
     cs[i & 1] = fmaxf(cs[i & 1], __uint_as_float(us[i]));
     cd[i & 1] = fmaxf(cd[i & 1], __uint_as_float(ud[i]));
   }
-  const float ns = fmaxf(cs[0], cs[1]) * kLog2e, nd = fmaxf(cd[0], cd[1]) * kLog2e;
+  const float ns = fmaxf(cs[0], cs[1]), nd = fmaxf(cd[0], cd[1]);
   if (ns > s.ms || nd > s.md) {
     const float ms = fmaxf(s.ms, ns), md = fmaxf(s.md, nd);
-    const float fs = kl_ex2(s.ms - ms), fd = kl_ex2(s.md - md);   // first chunk: the sums are 0, the factor 0
+    // a maximum that stays where it is (at -inf too) scales by 1; without one so far the sums are 0
+    const float fs = ms == s.ms ? 1.f : kl_ex2((s.ms - ms) * kLog2e), fd = md == s.md ? 1.f : kl_ex2((s.md - md) * kLog2e);
     s.zs *= fs;
     s.zd *= fd;
     s.x *= fd;
     s.ms = ms;
     s.md = md;
   }
-  // a maximum of -inf (every logit so far) subtracts nothing, so that the terms are 0
+  // a maximum of -inf (every logit so far) subtracts nothing, so that the exponentials are 0
   const float ms = s.ms == -INFINITY ? 0.f : s.ms, md = s.md == -INFINITY ? 0.f : s.md;
   const float2 l2 = make_float2(kLog2e, kLog2e), ms2 = make_float2(-ms, -ms), md2 = make_float2(-md, -md);
   const float2 minus = make_float2(-1.f, -1.f), zero = make_float2(0.f, 0.f);
@@ -98,7 +100,7 @@ __device__ __forceinline__ void kl_fold(KlSums& s, const uint32_t* us, const uin
 #pragma unroll
   for (int i = 0; i < 16; ++i) {
     const float2 a = f2(us[2 * i], us[2 * i + 1]), b = f2(ud[2 * i], ud[2 * i + 1]);
-    const float2 ta = __ffma2_rn(a, l2, ms2), tb = __ffma2_rn(b, l2, md2);
+    const float2 ta = __fmul2_rn(__fadd2_rn(a, ms2), l2), tb = __fmul2_rn(__fadd2_rn(b, md2), l2);
     const float2 e = make_float2(kl_ex2(tb.x), kl_ex2(tb.y));
     zs[i & 1] = __fadd2_rn(zs[i & 1], make_float2(kl_ex2(ta.x), kl_ex2(ta.y)));
     zd[i & 1] = __fadd2_rn(zd[i & 1], e);
@@ -305,7 +307,7 @@ __global__ void __launch_bounds__(256)
     double zs = 0.0, zd = 0.0, x = 0.0;
     for (int i = lane; i < n; i += 32) {
       const float* r = at(i);
-      const float fs = r[0] == ms ? 1.f : exp2f(r[0] - ms), fd = r[2] == md ? 1.f : exp2f(r[2] - md);
+      const float fs = r[0] == ms ? 1.f : expf(r[0] - ms), fd = r[2] == md ? 1.f : expf(r[2] - md);
       zs += (double)r[1] * fs;
       zd += (double)r[3] * fd;
       x += (double)r[4] * fd;
@@ -313,7 +315,7 @@ __global__ void __launch_bounds__(256)
     zs = warp_sum(zs);
     zd = warp_sum(zd);
     x = warp_sum(x);
-    if (lane == 0) mine += x / zd + log(zs / zd) + 0.69314718055994530942 * ((double)ms - (double)md);
+    if (lane == 0) mine += x / zd + log(zs / zd) + ((double)ms - (double)md);
   }
   if (lane == 0) red[warp] = mine;
   __syncthreads();

@@ -114,6 +114,60 @@ def test_align_output_tiles(A, n, d, V, scale):
     assert vals[0][0] == pytest.approx(ref.sum(), rel=1e-4)
 
 
+@pytest.mark.parametrize("at", [0, 32, 96, 128, 160])
+@pytest.mark.parametrize("mask", ["student_inf", "student_lowest", "student_1e30", "both_lowest"])
+def test_align_output_masked_classes(A, mask, at):
+    """bf16: 32 classes masked by logits at the lowest finite value or past it
+    (-inf, by overflow of the sum), at every place of a chunk in its tile. A class
+    that the dense model allows and the student gives -inf makes the loss +inf (the
+    student's lowest values too, or near 1e39: a row's fp32 sum of them may
+    overflow); at -1e30 they dominate it, in both models at once they drop out.
+    (fp32 sums: 1e-4 of the value, as for the tiles.)"""
+    g = np.random.default_rng(at)
+    n, d, V = 70, 64, 192
+    lowest = float(torch.finfo(torch.bfloat16).min)
+    hs = S.round_to(g.standard_normal((n, d)).astype(np.float32), "bf16")
+    hd = S.round_to((hs + 0.3 * g.standard_normal((n, d))).astype(np.float32), "bf16")
+    W = S.round_to((g.standard_normal((V, d)) / np.sqrt(d)).astype(np.float32), "bf16")
+    W[:, 0] = 0.0
+    W[at:at + 32] = 0.0
+    W[at:at + 32, 0] = 2.0 if mask == "student_inf" else 1.0
+    hs[:, 0] = S.round_to(np.float32([-1e30]), "bf16")[0] if mask == "student_1e30" else lowest
+    hd[:, 0] = lowest if mask == "both_lowest" else 0.0
+    acc = torch.zeros(2, dtype=torch.float64, device="cuda")
+    ws = A.workspace(A.lib().adadsf_align_workspace_size(n, V))
+    A.adadsf_align_output(*(H.to_dev(a, torch.bfloat16) for a in (hs, hd, W)), acc, ws=ws)
+    assert A.adadsf_sync_check(ws) == A.OK
+    got = float(acc[0])
+    if mask in ("student_inf", "student_lowest"):
+        assert got == np.inf if mask == "student_inf" else got > 1e37
+        return
+    ls, ld = (h.astype(np.float64) @ W.astype(np.float64).T for h in (hs, hd))
+    lse = lambda l: l.max(1, keepdims=True) + np.log(np.exp(l - l.max(1, keepdims=True)).sum(1, keepdims=True))
+    lps, lpd = ls - lse(ls), ld - lse(ld)
+    ref = float((np.exp(lpd) * (lpd - lps)).sum())
+    assert np.isfinite(got) and got == pytest.approx(ref, rel=1e-4)
+
+
+def test_align_output_many_row_blocks(A):
+    """bf16, 64 classes: a tile a row block, and more than two row blocks for
+    every CTA of the persistent grid. Loss of each quarter of the rows against its
+    own call."""
+    n = 2 * 128 * torch.cuda.get_device_properties(0).multi_processor_count + 200
+    n -= n % 4
+    g = torch.Generator(device="cuda").manual_seed(n)
+    rnd = lambda *shape: torch.randn(shape, generator=g, device="cuda")
+    hd = rnd(n, 64)
+    hs, hd, W = (hd + 0.3 * rnd(n, 64)).bfloat16(), hd.bfloat16(), (rnd(64, 64) / 8).bfloat16()
+    acc = torch.zeros(2, dtype=torch.float64, device="cuda")
+    ws = A.workspace(A.lib().adadsf_align_workspace_size(n, 64))
+    A.adadsf_align_output(hs, hd, W, acc, ws=ws)
+    assert A.adadsf_sync_check(ws) == A.OK
+    ls, ld = (torch.log_softmax(h.double() @ W.double().T, -1) for h in (hs, hd))
+    ref = (ld.exp() * (ld - ls)).sum().item()
+    assert acc[1].item() == n and acc[0].item() == pytest.approx(ref, rel=1e-5)
+
+
 QWEN_SMALL = S.QWEN25_1_5B.replace(d=1024, n_heads=8, n_kv_heads=2, ffn=1536, n_layers=1)
 
 
