@@ -282,41 +282,56 @@ __global__ void __launch_bounds__(kKlThreads, 1)
   }
 }
 
-// The records of each row (one warp per row) into its KL, then one double per
-// block, in a fixed order. A half without a class (ms = md = -inf, sums 0) adds nothing.
+// The records of each row into its KL, L lanes a row (the other lanes of a warp take
+// other rows), then one double per block, in a fixed order. A half without a class (ms =
+// md = -inf, sums 0) adds nothing.
+// L = 1 or 32: an instruction in fp64 takes the SM as long for one lane as for 32, so
+// that a lane a row does the division and logarithm of 32 rows at once, and its walk
+// along the records is no longer than a warp's sum over its lanes while there are
+// few. In all, us, warp / lane a row: 40,000 rows of 64 classes (2 to 6 records) 196 / 25,
+// 20,000 of 1024 135 / 49, 4096 of 50304 (up to 12) 321 / 309, 2000 of 50304 (22) 168 / 173,
+// 1000 of 50304 (42) 90 / 112 (d = 512).
+constexpr int kKlFewRecords = 16;
+
+template <int L>
 __global__ void __launch_bounds__(256)
     kl_merge_kernel(const float* rec, int M, int num_n, int64_t tiles, int G, double* partials) {
   pdl_wait();
   pdl_trigger();
   __shared__ double red[8];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int ROWS = 256 / L;   // rows a block takes at once
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, li = threadIdx.x % L;
   double mine = 0.0;
-  for (int64_t m = (int64_t)blockIdx.x * 8 + warp; m < M; m += (int64_t)gridDim.x * 8) {
+  for (int64_t m = (int64_t)blockIdx.x * ROWS + threadIdx.x / L; m < M; m += (int64_t)gridDim.x * ROWS) {
     const int64_t mb = m / kKlM;
     const int n = 2 * (kl_owner(tiles, G, (mb + 1) * num_n - 1) - kl_owner(tiles, G, mb * num_n) + 1);
     auto at = [&](int i) { return rec + (((int64_t)(i >> 1) * M + m) * 2 + (i & 1)) * kKlRec; };
     float ms = -INFINITY, md = -INFINITY;
-    for (int i = lane; i < n; i += 32) {
+    for (int i = li; i < n; i += L) {
       ms = fmaxf(ms, at(i)[0]);
       md = fmaxf(md, at(i)[2]);
     }
-    for (int o = 16; o > 0; o >>= 1) {
-      ms = fmaxf(ms, __shfl_xor_sync(0xffffffffu, ms, o));
-      md = fmaxf(md, __shfl_xor_sync(0xffffffffu, md, o));
-    }
+    if (L == 32)
+      for (int o = 16; o > 0; o >>= 1) {
+        ms = fmaxf(ms, __shfl_xor_sync(0xffffffffu, ms, o));
+        md = fmaxf(md, __shfl_xor_sync(0xffffffffu, md, o));
+      }
     double zs = 0.0, zd = 0.0, x = 0.0;
-    for (int i = lane; i < n; i += 32) {
+    for (int i = li; i < n; i += L) {
       const float* r = at(i);
       const float fs = r[0] == ms ? 1.f : expf(r[0] - ms), fd = r[2] == md ? 1.f : expf(r[2] - md);
       zs += (double)r[1] * fs;
       zd += (double)r[3] * fd;
       x += (double)r[4] * fd;
     }
-    zs = warp_sum(zs);
-    zd = warp_sum(zd);
-    x = warp_sum(x);
-    if (lane == 0) mine += x / zd + log(zs / zd) + ((double)ms - (double)md);
+    if (L == 32) {
+      zs = warp_sum(zs);
+      zd = warp_sum(zd);
+      x = warp_sum(x);
+    }
+    if (li == 0) mine += x / zd + log(zs / zd) + ((double)ms - (double)md);
   }
+  if (L == 1) mine = warp_sum(mine);   // L == 32: lane 0 has the warp's
   if (lane == 0) red[warp] = mine;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -352,9 +367,14 @@ cudaError_t kl_tc(const void* hs, const void* hd, const void* w, int64_t n_rows,
   const int G = (int)std::min<int64_t>(tiles, dev.num_sms);
   e = launch_pdl(kl_tc_kernel, dim3((unsigned)G), dim3(kKlThreads), kKlSmem, dev.stream, ts, td, tw, p);
   if (e != cudaSuccess) return e;
-  const int nb = train_row_blocks(n_rows);
-  e = launch_pdl(kl_merge_kernel, dim3((unsigned)nb), dim3(256), 0, dev.stream, (const float*)rec, p.M, p.num_n, tiles, G,
-                 partials);
+  // records of a row, at most: the CTAs whose ranges a row block's tiles touch, two each
+  const int64_t records = 2 * std::min<int64_t>(G, p.num_n / (tiles / G) + 2);
+  const bool few = records <= kKlFewRecords;
+  const int nb = few ? (int)std::min<int64_t>(train_row_blocks(n_rows), (n_rows + 255) / 256) : train_row_blocks(n_rows);
+  e = few ? launch_pdl(kl_merge_kernel<1>, dim3((unsigned)nb), dim3(256), 0, dev.stream, (const float*)rec, p.M, p.num_n,
+                       tiles, G, partials)
+          : launch_pdl(kl_merge_kernel<32>, dim3((unsigned)nb), dim3(256), 0, dev.stream, (const float*)rec, p.M, p.num_n,
+                       tiles, G, partials);
   if (e != cudaSuccess) return e;
   return sum_partials(partials, nb, n_rows, acc, dev);
 }
