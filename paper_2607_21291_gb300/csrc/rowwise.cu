@@ -675,7 +675,6 @@ __global__ void __launch_bounds__(kSelThreads)
 }
 
 // ---------------------------------------------------------------- Eq. 4 statistics
-constexpr int kStatThreads = 256;
 constexpr int kStatRows = 32;   // rows a block sums at a time
 
 // The fp64 part of Eq. 4 for a block's kStatRows rows at once, one row a lane of
@@ -706,15 +705,18 @@ __device__ __forceinline__ void cos_store(const double (&acc)[3], double* partia
   }
 }
 
-// Eq. 4 sums over rows: a warp takes four rows at once (fp32 sums a.b, |a|^2,
-// |b|^2), then the fp64 part over the block's 32 rows.
-template <typename T>
-__global__ void __launch_bounds__(kStatThreads) cos_rows_kernel(const T* a, const T* b,
-                                                                int64_t n_rows, int d, int mode,
-                                                                double* partials) {
+// Eq. 4 sums over rows: a warp takes R rows at once (fp32 sums a.b, |a|^2,
+// |b|^2), then the fp64 part over the block's 32 rows. R = 4 keeps eight loads a lane
+// in flight; with no more blocks than SMs a warp per row (R = 1) does it sooner. us from a
+// cold L2, R = 4 / 1: 300 x 3584 29.9 / 20.6, 1000 x 768 15.5 / 14.5, 4864 x 3584 37.0 / 28.8,
+// 5000 x 3584 37.0 / 38.1, 8192 x 768 17.6 / 20.6.
+template <typename T, int R>
+__global__ void __launch_bounds__(32 * kStatRows / R) cos_rows_kernel(const T* a, const T* b,
+                                                                      int64_t n_rows, int d, int mode,
+                                                                      double* partials) {
   pdl_wait();
   pdl_trigger();
-  constexpr int V = Elem<T>::kVec, R = kStatRows / (kStatThreads / 32);
+  constexpr int V = Elem<T>::kVec;
   __shared__ float sums[kStatRows][3];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   double acc[3] = {0, 0, 0};
@@ -1131,19 +1133,22 @@ int stats_partials_count(int64_t n_rows) {
   return (int)(want < cap ? (want > 0 ? want : 1) : cap);
 }
 
+template <typename T>
+static cudaError_t cos_rows(const T* a, const T* b, int64_t n_rows, int d, int mode, double* partials, const Dev& dev) {
+  const int nb = stats_partials_count(n_rows);
+  return nb <= dev.num_sms ? launch_pdl(cos_rows_kernel<T, 1>, dim3(nb), dim3(32 * kStatRows), 0, dev.stream, a, b, n_rows,
+                                        d, mode, partials)
+                           : launch_pdl(cos_rows_kernel<T, 4>, dim3(nb), dim3(8 * kStatRows), 0, dev.stream, a, b, n_rows, d,
+                                        mode, partials);
+}
+
 cudaError_t cos_stats(int dtype, const void* a, const void* b, int64_t n_rows, int d, int mode,
                       double* partials, double* acc, const Dev& dev) {
   if (n_rows <= 0) return cudaSuccess;
-  const int nb = stats_partials_count(n_rows);
-  cudaError_t e;
-  if (dtype == kBF16)
-    e = launch_pdl(cos_rows_kernel<bf16>, dim3(nb), dim3(kStatThreads), 0, dev.stream,
-                   static_cast<const bf16*>(a), static_cast<const bf16*>(b), n_rows, d, mode, partials);
-  else
-    e = launch_pdl(cos_rows_kernel<float>, dim3(nb), dim3(kStatThreads), 0, dev.stream,
-                   static_cast<const float*>(a), static_cast<const float*>(b), n_rows, d, mode,
-                   partials);
+  const cudaError_t e = dtype == kBF16 ? cos_rows(static_cast<const bf16*>(a), static_cast<const bf16*>(b), n_rows, d, mode, partials, dev)
+                                       : cos_rows(static_cast<const float*>(a), static_cast<const float*>(b), n_rows, d, mode, partials, dev);
   if (e != cudaSuccess) return e;
+  const int nb = stats_partials_count(n_rows);
   return launch_pdl(cos_finish_kernel, dim3(1), dim3(256), 0, dev.stream, partials, nb, n_rows, mode,
                     acc);
 }

@@ -502,12 +502,15 @@ def test_layer_stats(A, n, d, dtype):
     assert again.cpu().numpy().tolist() == got.tolist()  # bit-reproducible
 
 
-@pytest.mark.parametrize("n,d,dtype", [(31, 8, "bf16"), (32, 264, "bf16"), (33, 4, "f32"), (70001, 72, "bf16")])
+@pytest.mark.parametrize("n,d,dtype", [(31, 8, "bf16"), (32, 264, "bf16"), (33, 4, "f32"), (0, 2048, "bf16"), (1, 516, "f32"),
+                                       (70001, 72, "bf16")])
 def test_layer_stats_row_groups(A, n, d, dtype):
-    """Rows summed 32 at a time: last groups short, full and of one row, and more
-    groups than blocks. A row's fp32 sums hold d / 32 + 5 roundings at most, a
+    """Rows summed 32 at a time: last groups short, full and of one row, as many
+    groups as SMs and one more (n 0 and 1: the last that takes a warp per row, and
+    the first that does not), and more groups than blocks. A row's fp32 sums hold d / 32 + 5 roundings at most, a
     cosine three such sums, so well under 1e-5 each; the sum over rows is fp64."""
     td = torch.bfloat16 if dtype == "bf16" else torch.float32
+    n += 32 * torch.cuda.get_device_properties(0).multi_processor_count if n < 2 else 0
     gen = torch.Generator(device="cuda").manual_seed(n)
     a = torch.randn((n, d), generator=gen, device="cuda").to(td)
     b = (a.float() + 0.7 * torch.randn((n, d), generator=gen, device="cuda")).to(td)
