@@ -432,9 +432,12 @@ def test_attention(A, hq, hkv, hd, B, K, dtype):
         assert H.max_rel(got[b * K:(b + 1) * K], ref) < (2e-2 if dtype == "bf16" else 1e-5)
 
 
-@pytest.mark.parametrize("hq,hkv,hd,B,K", [(8, 8, 64, 1, 65), (8, 2, 64, 3, 128), (2, 1, 128, 2, 383), (1, 1, 64, 1, 700)])
+@pytest.mark.parametrize("hq,hkv,hd,B,K", [(8, 8, 64, 1, 65), (8, 2, 64, 3, 128), (2, 1, 128, 2, 383), (1, 1, 64, 1, 700),
+                                           (8, 2, 64, 1, 8), (8, 2, 64, 1, 9), (8, 2, 64, 40, 16), (8, 8, 64, 40, 17),
+                                           (2, 1, 128, 3, 1), (16, 4, 128, 30, 13)])
 def test_attention_f32_tiles(A, hq, hkv, hd, B, K):
-    """Key and query tiles of 64 of the fp32 kernel, and causality to the bit: an
+    """Key and query tiles of 64 of the fp32 kernel, both sides of the lines to the
+    one for short sequences (8 keys, 16 with many heads), and causality to the bit: an
     infinite value and a NaN key of the last token leave every earlier row as it
     was. fp32 softmax and sums over K keys: within 1e-5 of the largest element."""
     shape = S.PYTHIA_160M.replace(n_heads=hq, n_kv_heads=hkv, head_dim=hd, d=hq * hd, dtype="f32")
