@@ -245,7 +245,7 @@ void carve_layer(const adadsf_model_cfg* c, int B, int T, int K, Carver& cv, Lay
   // value heads transposed for the tensor-core attention: [B][Hkv][hd][vt_pad(K)]
   s.vt = c->dtype == ADADSF_BF16 ? cv.take((size_t)B * kv * vt_pad(K) * es) : 0;
   s.attn = cv.take(M * q * es);
-  s.ao = cv.take(M * c->d * es);
+  s.ao = c->arch == ADADSF_ARCH_QWEN ? cv.take(M * c->d * es) : 0;   // h = x + O W_o^T
   s.act = cv.take(M * c->ffn * es);
   // fp32 partial tiles of projections split along K (tensor-core path)
   s.split = c->dtype == ADADSF_BF16 ? cv.take(gemm_split_scratch_bytes()) : 0;

@@ -101,6 +101,18 @@ def test_alloc_rejects_bad_args(A):
         A.adadsf_alloc_ratios([0.5, 0.6], 0.5, tau=0.0)
 
 
+def test_neox_layer_workspace_is_what_it_writes(A):
+    """A fp32 GPT-NeoX layer stores scores, kept positions, both norms, QKV,
+    attention and MLP rows (the output projection goes into the residual's sum):
+    the workspace holds these, each on a 256-byte boundary, the error word, the
+    counters and the rotary table, and nothing else."""
+    s, (B, T, K) = S.PYTHIA_70M, (3, 100, 37)
+    M = B * K
+    parts = [256, 16384, T * (s.rotary_dim // 2) * 8, B * T * 4, M * 4, M * 4, M * s.d * 4, M * s.d * 4,
+             M * s.qkv_dim * 4, M * s.q_dim * 4, M * s.ffn * 4]
+    assert A.adadsf_layer_workspace_size(A.make_cfg(s), B, T, K) == sum((p + 255) // 256 * 256 for p in parts)
+
+
 def test_workspace_sizes(A):
     for key in ("c1", "c2", "c3", "c4", "c5"):
         wl = S.WORKLOADS[key]
