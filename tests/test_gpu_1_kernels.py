@@ -113,8 +113,9 @@ def test_linear_bf16(A, M, N, Kd, act):
                                         (1024, 768, 768, 1), (1024, 768, 3072, 0), (333, 640, 960, 1),
                                         (129, 128, 192, 0),
                                         # fewer than 128 rows: a stage loads only them, rounded up to 8
-                                        (5, 512, 3584, 0), (13, 4608, 3584, 1), (16, 3584, 18944, 0),
-                                        (17, 1024, 2048, 1), (100, 640, 1536, 0)])
+                                        (9, 8192, 2048, 1), (17, 1024, 2048, 1), (40, 4608, 3584, 1), (100, 640, 1536, 0),
+                                        # 16 rows and fewer: direct and streamed products, which never split into scratch
+                                        (5, 512, 3584, 0), (13, 4608, 3584, 1), (16, 3584, 18944, 0)])
 def test_linear_bf16_small_m(A, M, N, Kd, act):
     """Small-M projections of the sparse layers: one wave of tiles, long K
     (with room for scratch most of these run split along K over clusters of 2
@@ -169,13 +170,18 @@ def test_linear_bf16_few_rows(A, M, N, Kd, act):
     assert bool((out[M] == 7.0).all())          # nothing past the last row
 
 
-@pytest.mark.parametrize("M,N,Kd,act", [(1, 3584, 4096, 0), (8, 3584, 3968, 1), (9, 1088, 8256, 0), (16, 4864, 1728, 1),
-                                        (16, 4928, 1728, 0), (13, 512, 16448, 0), (16, 448, 20480, 0)])
+@pytest.mark.parametrize("M,N,Kd,act", [(1, 3584, 4096, 0), (8, 3584, 3968, 1), (9, 1088, 8256, 0), (16, "last", 1728, 1),
+                                        (16, "past", 1728, 0), (13, 512, 16448, 0), (16, 448, 20480, 0), (1, 512, 27392, 0),
+                                        (7, "last", 3136, 1)])
 def test_linear_bf16_few_rows_streamed(A, M, N, Kd, act):
     """At most 16 rows and more weights than the direct kernel takes: one and two
-    8-row halves, 1 to 8 groups of columns a pair of CTAs, K of an odd number of 64-element
-    blocks (and N past either end of the range, the tensor-core kernels). One bf16
-    rounding of the output (2^-9 of an element, under 8e-3 of the largest)."""
+    8-row halves, 1 to 8 groups of columns a pair of CTAs (up to 64 columns for
+    each pair of SMs: the last width of that, and one past it), K of an odd number
+    of 64-element blocks (and N past either end of the range, the tensor-core
+    kernels). One bf16 rounding of the output (2^-9 of an element, under 8e-3 of the
+    largest)."""
+    pairs = torch.cuda.get_device_properties(0).multi_processor_count // 2
+    N = {"last": 64 * pairs, "past": 64 * (pairs + 1)}.get(N, N)
     g = torch.Generator(device="cuda").manual_seed(N + Kd)
     rnd = lambda *shape: torch.randn(shape, generator=g, device="cuda")
     x, w, b = rnd(M, Kd).bfloat16(), (rnd(N, Kd) / Kd ** 0.5).bfloat16(), rnd(N).bfloat16()
@@ -344,11 +350,13 @@ def test_router(A, shape, n):
     assert err < (5e-3 if shape.dtype == "bf16" else 1e-5)
 
 
-@pytest.mark.parametrize("shape,n", [(S.PYTHIA_160M, 2048), (S.PYTHIA_1_4B, 16384), (S.QWEN25_1_5B, 999),
+@pytest.mark.parametrize("shape,n", [(S.PYTHIA_160M, 2048), (S.PYTHIA_160M, 2600), (S.PYTHIA_1_4B, 16384),
+                                     (S.QWEN25_1_5B, 999), (S.QWEN25_1_5B, 3001),
                                      (S.QWEN25_7B.replace(ffn=256), 4096),
                                      (S.QWEN25_7B.replace(ffn=256), 25600 - 77)])
 def test_router_split(A, shape, n):
-    """Router with room for scratch. Up to one wave of 128-token tiles every
+    """Router with room for scratch. Up to 16 tokens an SM (2048 and 999 here)
+    it is not used. Past that and up to one wave of 128-token tiles every
     CTA takes whole tiles; past it (the last case: 200 tiles of d = 3584 on
     the GPU's ~150 SMs) the CTAs take equal ranges of k-blocks, tiles are
     split along d and the last CTA of a tile sums the partials in a fixed

@@ -143,11 +143,13 @@ def _prefill_then_decode(A, shape, B, T0, K, steps, C_max, gated, etol, folded=F
             assert (counts[l] == 0).all()
 
 
-def test_decode_step_in_a_cuda_graph(A):
+@pytest.mark.parametrize("B", [2, 18])
+def test_decode_step_in_a_cuda_graph(A, B):
     """A decode step reads its position and counts from the cache, so one
-    captured graph replays step after step: the same outputs as eager steps."""
+    captured graph replays step after step: the same outputs as eager steps (with
+    18 sequences the graph holds the second stream's part too)."""
     shape = NEOX_SMALL
-    B, T0, C_max, K = 2, 48, 64, [24, 48, 12]
+    T0, C_max, K = 48, 64, [24, 48, 12]
     td = H.tdtype(shape)
     hostL = [H.host_layer(shape, 21, l) for l in range(shape.n_layers)]
     model = A.DeviceModel(A.make_cfg(shape), [A.to_device(w, td) for w in hostL],
@@ -162,6 +164,7 @@ def test_decode_step_in_a_cuda_graph(A):
         tok = torch.empty(B, dtype=torch.int32, device="cuda")
         h = torch.empty((B, shape.d), dtype=td, device="cuda")
         stream = torch.cuda.Stream()
+        stream.wait_stream(torch.cuda.current_stream())
         res = []
         with torch.cuda.stream(stream):
             if use_graph:
@@ -262,27 +265,38 @@ def _decode_run(A, model, td, ids, B, T0, K, C_max, steps, stream, capture_first
     return torch.stack(out)
 
 
-def test_decode_captured_before_any_eager_step(A):
-    """A step captured into a graph before any uncaptured step on its stream
-    runs on that stream alone (keep decision inside the norm launch); its
-    outputs equal those of eager steps, which fork the router onto a second
-    stream."""
+@pytest.mark.parametrize("B", [2, 17])
+def test_decode_captured_before_any_eager_step(A, B):
+    """A step of more than 16 sequences captured into a graph before any
+    uncaptured step on its stream runs on that stream alone (keep decision inside
+    the norm launch); its outputs equal those of eager steps, which fork the router
+    onto a second stream (a router launch of its own). At most 16 sequences take one
+    stream either way (router, decision and norm in one launch). The captured
+    stream is of high priority: no other test has made a step on one."""
     shape = QWEN_SMALL
     model, td = _small_model(A, shape, 61)
-    B, T0, C_max, K = 2, 96, 112, [48, 30, 96]
+    T0, C_max, K = 96, 112, [48, 30, 96]
     ids = torch.from_numpy(S.token_ids(62, B, T0 + 4, shape.vocab)).cuda()
     eager = _decode_run(A, model, td, ids, B, T0, K, C_max, 4, torch.cuda.Stream())
-    graph = _decode_run(A, model, td, ids, B, T0, K, C_max, 4, torch.cuda.Stream(), capture_first=True)
+    graph = _decode_run(A, model, td, ids, B, T0, K, C_max, 4, torch.cuda.Stream(priority=-1), capture_first=True)
     assert torch.equal(eager, graph)
+    cache, tok = A.kv_cache(model.cfg, B, C_max), ids[:, 0].contiguous()
+    h = torch.empty((B, shape.d), dtype=td, device="cuda")
+    A.adadsf_prefill(model, ids[:, :T0].contiguous(), K, torch.empty((B, T0, shape.d), dtype=td, device="cuda"), cache, C_max)
+    A.adadsf_profile_begin(256)
+    A.adadsf_decode_step(model, tok, h, cache, C_max)
+    kinds = {r[0] for r in A.adadsf_profile_end(256)}
+    assert "decide" in kinds and ("router" in kinds) == (B > 16), kinds
 
 
-def test_decode_on_two_streams_interleaved(A):
+@pytest.mark.parametrize("B", [2, 20])
+def test_decode_on_two_streams_interleaved(A, B):
     """Two models decode on two streams with their steps enqueued in turn:
-    each gets the outputs it gets alone (each caller stream has its own
-    second stream and fork / join events)."""
+    each gets the outputs it gets alone (past 16 sequences each caller stream has
+    its own second stream and fork / join events)."""
     shape = NEOX_SMALL
     (m1, td), (m2, _) = _small_model(A, shape, 71), _small_model(A, shape, 72)
-    B, T0, C_max, K, steps = 2, 64, 80, [40, 64, 20], 4
+    T0, C_max, K, steps = 64, 80, [40, 64, 20], 4
     ids1 = torch.from_numpy(S.token_ids(73, B, T0 + steps, shape.vocab)).cuda()
     ids2 = torch.from_numpy(S.token_ids(74, B, T0 + steps, shape.vocab)).cuda()
     alone1 = _decode_run(A, m1, td, ids1, B, T0, K, C_max, steps, torch.cuda.Stream())
