@@ -6,17 +6,19 @@
 // 128 weight rows, partial tiles exchanged between the CTAs of a split): a few MB of
 // weights took 8 to 15 us. Here a block takes 8-row groups of W, as evenly as the
 // groups divide, its 16 warps every sixteenth 64-byte piece of K, and the first pieces
-// are on their way before the block waits for the previous kernel (which is one of
-// the same call, so that weights do not depend on it). The product is warp-level (mma.sync m16n8k16): 16 weight rows
-// are the A operand, the rows of A the B operand's columns. Both come straight from
-// memory: a lane loads 16 consecutive bytes of a row, and since the order of k inside
+// are on their way before the block waits for the previous kernel (behind a launch of
+// the same call, so that the weights do not depend on it; the first launch of a call
+// waits before it reads them, 0.4 to 0.8 us more in a row of products). The product is
+// warp-level (mma.sync m16n8k16): 16 weight rows are the A operand, the rows of A the
+// B operand's columns. Both come straight from memory: a lane loads 16 consecutive bytes of a row, and since the order of k inside
 // a product is free as long as both operands agree, those bytes are the fragment as
 // they come. The warps' sums are added in warp order through shared memory
 // (bit-reproducible), and the next tile's first pieces load meanwhile.
 //
 // Its line lies at the weights' size (MB), 28 up to 8 rows and 16 above: larger
 // weights stream faster by TMA, whose boxes keep more in flight than 16 loads a lane (the second
-// kernel below, or the tensor-core kernels). us per product from a cold L2, there / here:
+// kernel below, or the tensor-core kernels). us per product from a cold L2, weights
+// requested ahead, tensor-core kernels / here:
 //   N x K            MB     1 row          16 rows
 //   768 x 768        1.2    5.3 / 2.1      5.1 / 2.9
 //   2304 x 768       3.5    5.4 / 2.5      5.4 / 3.2
@@ -251,16 +253,25 @@ __device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v) {
 // tensor-core kernels, whose tiles of 128 weight rows and splits of 2 or 4 fill 112 to
 // 144 of the SMs, the groups divide over pairs of CTAs, each CTA half of K, so
 // that every SM streams and only one partial tile passes between two CTAs. A thread
-// brings stages of 128 k, one box of W (a tile's rows, two blocks of 128-byte swizzled
-// rows) and one of A, into a ring of 170 KB; each of eight warps takes one 16-k product of a
-// stage (mma.sync: 24 of them a stage at 48 rows, far from a limit). The sums
+// brings stages of 128 k, one box of W (U groups of 8 rows, two blocks of 128-byte swizzled
+// rows) and one of A (NT groups), 2 KB a group, into a ring of up to 12 stages and 184 KB;
+// each of eight warps takes one 16-k product of a stage (mma.sync: 4 U NT of them a
+// stage for all, at most 64, far from a limit). The sums
 // of the warps are added in warp order, the pair's halves exchange theirs and
 // each finishes half of the outputs. One box of 8 rows each instead of one a stage: 47 us
-// at 3584 x 18944, TMA-issue bound, to 29. Chains of products of different weights, us
-// each at 16 rows, tensor-core kernels / here: 3584 x 18944 29.2 / 26.0, 4608 x 3584
-// 10.5 / 9.5, 2048 x 8192 12.9 / 13.0, 3584 x 3584 9.5 / 9.3, 4864 x 2048 8.4 / 7.8; 16
-// sequences at the Qwen2.5-7B shape, two layers, 16 steps 4241 -> 4084 us. With
-// more rows than one tile of 64 a pair (N > 4864) the exchanges and the repeated rows of A
+// at 3584 x 18944, TMA-issue bound, to 29. Chains of products of different weights,
+// requested ahead as inside a step, us each, tensor-core kernels / here:
+//   N x K            MB     1 row          8 rows         16 rows
+//   512 x 28672      29.4   31.4 / 28.5    31.5 / 28.6    31.4 / 29.7
+//   1024 x 16384     33.6   20.2 / 18.0    20.3 / 18.2
+//   2048 x 8192      33.6   13.2 / 12.2    13.1 / 12.3    13.1 / 12.7
+//   2048 x 11008     45.1   15.9 / 15.2    16.0 / 15.3    16.0 / 15.7
+//   3584 x 3584      25.7                                 9.6 / 9.4
+//   4608 x 3584      33.0   10.7 / 9.4     10.8 / 9.5     10.8 / 9.9
+//   3584 x 18944     136    29.5 / 25.9    29.7 / 26.4    29.8 / 26.8
+//   4864 x 8192      79.7   21.4 / 16.6    21.6 / 16.9    21.8 / 17.3
+// 16 sequences at the Qwen2.5-7B shape, two layers, 16 steps 4241 -> 4084 us. With
+// more rows than one tile of 64 a pair of SMs the exchanges and the repeated rows of A
 // lose: 8192 x 2048 12.5 / 14.5, 18944 x 3584 29 / 37, which stay where they were.
 // tmW2 / tmX2: the second K source.
 template <int NT>
@@ -461,9 +472,9 @@ double weight_bytes(const GemmArgs& g) {
 // Weights (bytes) up to which the first kernel is the faster one.
 double rows_line(const GemmArgs& a) { return a.M <= 8 ? 28e6 : 16e6; }
 
-// Products for the streaming kernel: more weights than that, one tile a pair of CTAs. From
-// 512 columns on it is the faster one (512 x 20480 23.4 us by the tensor-core kernels, 22.7 here);
-// below, too few pairs of CTAs have a group.
+// Products for the streaming kernel: more weights than that, one tile a pair of CTAs (64
+// columns a pair of SMs). From 512 columns on it is the faster one (512 x 28672 31.4 us by the
+// tensor-core kernels, 29.7 here); below, too few pairs of CTAs have a group.
 bool streams(const GemmArgs& a, int num_sms) {
   return a.epi.act != ACT_SWIGLU && a.K % 64 == 0 && a.K2 % 64 == 0 && a.N >= 512 &&
          a.N / 8 <= kGsGroups * (num_sms / 2) &&
