@@ -37,23 +37,6 @@ struct AttnF32 {
   static constexpr int SMEM = FLOATS * 4;
 };
 
-__device__ __forceinline__ void cp_async16_zfill(uint32_t dst, const void* src, bool valid) {
-  const int bytes = valid ? 16 : 0;   // 0: fill with zeros, nothing read
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
-}
-
-// Sum and maximum over the 16 threads that share a query row.
-__device__ __forceinline__ float max16(float v) {
-#pragma unroll
-  for (int o = 8; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-__device__ __forceinline__ float sum16(float v) {
-#pragma unroll
-  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 template <int HD>
 __global__ void __launch_bounds__(kAtThreads) attn_f32_kernel(const float* qkv, int64_t ldq, float* out, int64_t ldo,
                                                               int K, int n_heads, int n_kv, int B, float scale) {
@@ -79,7 +62,7 @@ __global__ void __launch_bounds__(kAtThreads) attn_f32_kernel(const float* qkv, 
       const int v = i * kAtThreads + tid;
       const int r = v / (HD / 4), c = (v % (HD / 4)) * 4;
       const bool ok = r0 + r < K;
-      cp_async16_zfill(smem_u32(dst + r * ld + c), base + (int64_t)(ok ? r0 + r : 0) * ldq + c0 + c, ok);
+      cp_async16(smem_u32(dst + r * ld + c), base + (int64_t)(ok ? r0 + r : 0) * ldq + c0 + c, ok);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };

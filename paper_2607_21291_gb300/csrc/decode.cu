@@ -207,25 +207,7 @@ __global__ void __launch_bounds__(kDecThreads)
 //   online softmax per row (exp2; the 4 lanes of a quad share a row)
 //   O (16 x HD) += P (16 x 16, bf16) . V (16 x HD)   (ldmatrix.trans)
 // and the four warps' (max, sum, O) merge in shared memory at the end.
-__device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t (&r)[4]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(addr));
-}
-__device__ __forceinline__ void ldsm_x4_t(uint32_t addr, uint32_t (&r)[4]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(addr));
-}
-// D += A . B for one m16n8k16 tile (A row-major 16 x 16, B column-major 16 x 8).
-__device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
-                                               uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
-      "{%8, %9}, {%0, %1, %2, %3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
+
 // Byte offset of (row, col) in a ring tile: boxes of 64 features (128 bytes)
 // side by side, each kDecTK rows of 128 bytes with the 16-byte chunks of a
 // row permuted by XOR with (row mod 8), as the TMA 128-byte swizzle writes them.
@@ -401,9 +383,9 @@ __global__ void __launch_bounds__(kDecTcThreads)
 #pragma unroll
       for (int ks = 0; ks < HD / 16; ++ks) {
         uint32_t kb[4];
-        ldsm_x4(kt + dec_swz(kw + (mi >> 1) * 8 + mr, ks * 16 + (mi & 1) * 8), kb);
-        mma_bf16_16816(sc[0], qa[ks], kb[0], kb[1]);
-        mma_bf16_16816(sc[1], qa[ks], kb[2], kb[3]);
+        ldmatrix_x4(kt + dec_swz(kw + (mi >> 1) * 8 + mr, ks * 16 + (mi & 1) * 8), kb);
+        mma_16816(sc[0], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], kb[0], kb[1]);
+        mma_16816(sc[1], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], kb[2], kb[3]);
       }
       // online softmax over the warp's 16 keys; key j0 + 8 nt + 2 tig + e
       const int j0 = lo + t * kDecTK + kw;
@@ -448,9 +430,9 @@ __global__ void __launch_bounds__(kDecTcThreads)
 #pragma unroll
       for (int np = 0; np < HD / 16; ++np) {
         uint32_t vb[4];
-        ldsm_x4_t(vt + dec_swz(kw + (mi & 1) * 8 + mr, np * 16 + (mi >> 1) * 8), vb);
-        mma_bf16_16816(o[2 * np], pa, vb[0], vb[1]);
-        mma_bf16_16816(o[2 * np + 1], pa, vb[2], vb[3]);
+        ldmatrix_x4_trans(vt + dec_swz(kw + (mi & 1) * 8 + mr, np * 16 + (mi >> 1) * 8), vb);
+        mma_16816(o[2 * np], pa[0], pa[1], pa[2], pa[3], vb[0], vb[1]);
+        mma_16816(o[2 * np + 1], pa[0], pa[1], pa[2], pa[3], vb[2], vb[3]);
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(empty0 + 8 * st);

@@ -68,15 +68,6 @@ __device__ __forceinline__ uint4 ld_w(const bf16* p) {
   return v;
 }
 
-__device__ __forceinline__ void mma_rows(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
-                                         uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
-      "{%8, %9}, {%0, %1, %2, %3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
 // Output element (row m of A, column n) from its sum (v2: the up weight's, DUAL).
 template <bool DUAL>
 __device__ __forceinline__ void rows_epilogue(const RowsDev& p, int m, int n, float v, float v2) {
@@ -186,8 +177,8 @@ __global__ void __launch_bounds__(kGrThreads, 1)
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) {
           const uint4 a = wc[u][0], b = wc[u][1], v = xv[u][nt];
-          mma_rows(acc[nt], a.x, b.x, a.y, b.y, v.x, v.y);
-          mma_rows(acc[nt], a.z, b.z, a.w, b.w, v.z, v.w);
+          mma_16816(acc[nt], a.x, b.x, a.y, b.y, v.x, v.y);
+          mma_16816(acc[nt], a.z, b.z, a.w, b.w, v.z, v.w);
         }
     }
     const Tile done = cur;
@@ -238,12 +229,6 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const void* tmap, int 
       " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
       "l"(reinterpret_cast<uint64_t>(tmap)), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
       : "memory");
-}
-__device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], uint32_t addr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(addr)
-               : "memory");
 }
 __device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
@@ -371,15 +356,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGsThreads, 1)
       if (!ok) break;
       const uint32_t base = ring + stage * stage_bytes;
       uint32_t xv[4];
-      ldmatrix_x4(xv, base + x_at);
+      ldmatrix_x4(base + x_at, xv);
 #pragma unroll
       for (int q = 0; q < kGsGroups / 2; ++q) {
         if (2 * q < cnt) {   // with an odd count the last 8 rows are others' bytes: their sums are dropped
           uint32_t wv[4];
-          ldmatrix_x4(wv, base + q * 2 * 1024 + w_at);
+          ldmatrix_x4(base + q * 2 * 1024 + w_at, wv);
 #pragma unroll
           for (int nt = 0; nt < NT; ++nt)
-            mma_rows(acc[q][nt], wv[0], wv[1], wv[2], wv[3], xv[2 * nt], xv[2 * nt + 1]);
+            mma_16816(acc[q][nt], wv[0], wv[1], wv[2], wv[3], xv[2 * nt], xv[2 * nt + 1]);
         }
       }
       __syncwarp();

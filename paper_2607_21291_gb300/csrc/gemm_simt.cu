@@ -72,11 +72,6 @@ struct F32Tile {
   static_assert((BM + BN) * 8 % THREADS == 0 && THREADS % 8 == 0, "loader");
 };
 
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {
-  const int bytes = valid ? 16 : 0;   // 0: fill with zeros, nothing read
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
-}
-
 // Rotary partner of columns n .. n + 3: 0 if they do not rotate, else the distance to
 // their pairs' other halves (the host fuses the rotation only where a half is whole
 // groups of four columns and both halves lie in one tile).

@@ -137,14 +137,7 @@ __device__ __forceinline__ float4 router_rows_units(const T* xr0, const T* xr1, 
 // from zero and added to the total in fp32, so that its truncating accumulator
 // never carries a long sum (the gradient's error against 64 bits is 1.4e-7 at 2048 rows
 // of 2048 features, 7.9e-7 as serial fp32 sums).
-__device__ __forceinline__ void mma_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
-                                          uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
-      "{%8, %9}, {%0, %1, %2, %3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
+//
 // One piece of 32 features of the operands, in flight.
 struct RouterPiece {
   uint4 w[8], xa, xb;
@@ -206,11 +199,16 @@ __device__ __forceinline__ float4 router_rows_partial(const bf16* xr0, const bf1
   return u;
 }
 
-// Sum over the 16 threads that share a row.
-__device__ __forceinline__ float row16_sum(float v) {
+// A row's score but for b2, from its units j0 ... j0 + 3 (u, no bias) in each of the 16
+// threads that share it.
+__device__ __forceinline__ float router_row_score(const float (&u)[4], int j0, const bf16* b1, const bf16* w2) {
+  float s = 0.f;
 #pragma unroll
-  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+  for (int e = 0; e < 4; ++e) {
+    const float v = u[e] + __bfloat162float(b1[j0 + e]);
+    s += __bfloat162float(w2[j0 + e]) * (v / (1.f + expf(-v)));
+  }
+  return sum16(s);
 }
 
 }  // namespace adadsf

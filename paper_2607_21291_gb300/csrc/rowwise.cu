@@ -279,13 +279,7 @@ __global__ void __launch_bounds__(kRrThreads)
       u[2] += f.z;
       u[3] += f.w;
     }
-    float s = 0.f;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float v = u[e] + __bfloat162float(rb1[j0 + e]);
-      s += __bfloat162float(w2[j0 + e]) * (v / (1.f + expf(-v)));
-    }
-    s = row16_sum(s);
+    const float s = router_row_score(u, j0, rb1, w2);
     if ((threadIdx.x & 15) == 0 && row < B) {
       scores[row] = s + __bfloat162float(rb2[0]);
       decide_row(row, scores, thr, hdr, C_max, lens, rows, pos, kept_out, err);
@@ -337,13 +331,7 @@ __global__ void __launch_bounds__(kRrThreads)
       u[2] += f.z;
       u[3] += f.w;
     }
-    float s = 0.f;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float v = u[e] + __bfloat162float(rb1[j0 + e]);
-      s += __bfloat162float(w2[j0 + e]) * (v / (1.f + expf(-v)));
-    }
-    s = row16_sum(s);
+    const float s = router_row_score(u, j0, rb1, w2);
     if ((threadIdx.x & 15) == 0 && r0 + row < n_rows) scores[r0 + row] = s + __bfloat162float(rb2[0]);
   }
   cluster_sync();   // the shares stay until the first CTA has read them
@@ -606,7 +594,7 @@ __global__ void __launch_bounds__(kRrThreads, 2)
       }
     }
   }
-  s = row16_sum(s);
+  s = sum16(s);
   if ((threadIdx.x & 15) == 0 && row < n) scores[row] = s + b2[0];
 }
 

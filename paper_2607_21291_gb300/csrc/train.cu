@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(kRrThreads, 2)
       dsi[e] = sg * (1.f + u * (1.f - sg)) * wj;   // w2 SiLU'(u), scaled by ds below
     }
   }
-  s = row16_sum(s) + Elem<T>::to_f(b2[0]);
+  s = sum16(s) + Elem<T>::to_f(b2[0]);
   const float sig = 1.f / (1.f + expf(-s));
   const float ds = sig * (1.f - sig) * gd_s[row];
   const int64_t m = m0 + row;
@@ -344,12 +344,6 @@ __global__ void __launch_bounds__(kRrThreads, 2)
   if (j0 == 0) ds_out[m] = ds;
 }
 
-__device__ __forceinline__ void ldsm_x4_trans(uint32_t addr, uint32_t (&r)[4]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(addr)
-               : "memory");
-}
 // f as a sum of three bf16 values (in the high halves of p): exact for finite f
 // (each part takes the next 8 significant bits), f itself rounded where it is not.
 __device__ __forceinline__ void bf16_parts(float f, uint32_t (&p)[3]) {
@@ -481,14 +475,14 @@ __global__ void __launch_bounds__(kRedThreads)
 #pragma unroll
         for (int q = 0; q < 2; ++q) {   // columns c0 + 16 q: rows ks + 8 (mi & 1), column chunk mi / 2
           const int r = ks + (mi & 1) * 8 + mr, c = (c0 >> 3) + 2 * q + (mi >> 1);
-          ldsm_x4_trans(sbase + 3 * PLANE + r * 128 + ((c ^ (r & 7)) << 4), b[q]);
+          ldmatrix_x4_trans(sbase + 3 * PLANE + r * 128 + ((c ^ (r & 7)) << 4), b[q]);
         }
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt) {
           uint32_t a[3][4];
           const int r = ks + (mi >> 1) * 8 + mr, c = (u0 >> 3) + 2 * mt + (mi & 1);
 #pragma unroll
-          for (int k = 0; k < 3; ++k) ldsm_x4_trans(sbase + k * PLANE + r * 128 + ((c ^ (r & 7)) << 4), a[k]);
+          for (int k = 0; k < 3; ++k) ldmatrix_x4_trans(sbase + k * PLANE + r * 128 + ((c ^ (r & 7)) << 4), a[k]);
 #pragma unroll
           for (int nt = 0; nt < 4; ++nt) {
             float p[4] = {0.f, 0.f, 0.f, 0.f};
