@@ -569,15 +569,8 @@ template <int HD>
 cudaError_t launch_attn(const void* qkv, int64_t ld_qkv, const void* vt, int pad, void* out,
                         int64_t ld_out, int B, int K, int Hq, int Hkv, const Dev& dev) {
   using C = AttnCfg<HD>;
-  static int attr_done[64] = {0};
-  int device = 0;
-  cudaGetDevice(&device);
-  if (device < 64 && !attr_done[device]) {
-    cudaError_t e = cudaFuncSetAttribute(attn_tc_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         C::SMEM);
-    if (e != cudaSuccess) return e;
-    attr_done[device] = 1;
-  }
+  const cudaError_t e = allow_smem<attn_tc_kernel<HD>, C::SMEM>();
+  if (e != cudaSuccess) return e;
   CUtensorMap tq, tv;
   if (!make_tmap_bf16(&tq, qkv, (uint64_t)B * K, (uint64_t)ld_qkv, (uint64_t)ld_qkv, 64, kQB) ||
       !make_tmap_bf16(&tv, vt, (uint64_t)B * Hkv * HD, (uint64_t)K, (uint64_t)pad, 64, HD))

@@ -1543,18 +1543,11 @@ template <int BN, bool DUAL, bool EXTRA>
 cudaError_t launch_x(const GemmArgs& a, const GemmArgs* b, const Dev& dev) {
   using C = TileCfg<BN, DUAL>;
   if (a.a_gather || (b && b->a_gather)) return cudaErrorInvalidValue;
-  static int attr_done[64] = {0};
-  int device = 0;
-  cudaGetDevice(&device);
-  if (device < 64 && !attr_done[device]) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<BN, DUAL, EXTRA>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
-    if (e != cudaSuccess) return e;
-    attr_done[device] = 1;
-  }
+  cudaError_t e = allow_smem<gemm_tc_kernel<BN, DUAL, EXTRA>, C::SMEM_BYTES>();
+  if (e != cudaSuccess) return e;
   CUtensorMap tm[4];
   GemmDev p, p2;
-  cudaError_t e = prepare<DUAL>(a, b, a_box_rows(a, b), BN, BN, dev, tm, p, p2);
+  e = prepare<DUAL>(a, b, a_box_rows(a, b), BN, BN, dev, tm, p, p2);
   if (e != cudaSuccess) return e;
   int64_t num_tiles = ((a.M + BM - 1) / BM) * ((a.N + p.bn - 1) / p.bn);
   if (b) num_tiles += ((b->M + BM - 1) / BM) * ((b->N + p2.bn - 1) / p2.bn);
@@ -1572,15 +1565,10 @@ cudaError_t launch(const GemmArgs& a, const GemmArgs* b, const Dev& dev) {
 template <int BN, bool DUAL, bool EXTRA>
 cudaError_t launch_pair_x(const GemmArgs& a, const GemmArgs* b, const Dev& dev) {
   using C = TileCfg<BN, DUAL, true>;
-  static int attr_done[64] = {0};
+  cudaError_t e = allow_smem<gemm_tc2_kernel<BN, DUAL, EXTRA>, C::SMEM_BYTES>();
+  if (e != cudaSuccess) return e;
   int device = 0;
   cudaGetDevice(&device);
-  if (device < 64 && !attr_done[device]) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_tc2_kernel<BN, DUAL, EXTRA>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
-    if (e != cudaSuccess) return e;
-    attr_done[device] = 1;
-  }
   // A persistent grid must not exceed the CTA pairs that can be resident at
   // once (a TPC with one SM unavailable cannot host a pair).
   static int max_pairs[64] = {0};
@@ -1590,7 +1578,7 @@ cudaError_t launch_pair_x(const GemmArgs& a, const GemmArgs* b, const Dev& dev) 
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = C::SMEM_BYTES;
     int n = 0;
-    cudaError_t e = cudaOccupancyMaxActiveClusters(&n, gemm_tc2_kernel<BN, DUAL, EXTRA>, &cfg);
+    e = cudaOccupancyMaxActiveClusters(&n, gemm_tc2_kernel<BN, DUAL, EXTRA>, &cfg);
     if (e != cudaSuccess || n <= 0) return e != cudaSuccess ? e : cudaErrorInvalidConfiguration;
     max_pairs[device] = n;
   }
@@ -1604,7 +1592,7 @@ cudaError_t launch_pair_x(const GemmArgs& a, const GemmArgs* b, const Dev& dev) 
     b_full = *b;
     b_full.tile_n = 0;
   }
-  cudaError_t e = prepare<DUAL>(a_full, b ? &b_full : nullptr, BM, BN, C::B_ROWS, dev, tm, p, p2);
+  e = prepare<DUAL>(a_full, b ? &b_full : nullptr, BM, BN, C::B_ROWS, dev, tm, p, p2);
   if (e != cudaSuccess) return e;
   int64_t num_tiles = ((a.M + 2 * BM - 1) / (2 * BM)) * ((a.N + BN - 1) / BN);
   if (b) num_tiles += ((b->M + 2 * BM - 1) / (2 * BM)) * ((b->N + BN - 1) / BN);
@@ -1625,18 +1613,12 @@ template <int BN>
 int sk_max_clusters(int S, const Dev& dev) {
   using C = TileCfg<BN, false>;
   static int cache[64][5] = {};
-  static int attr_done[64] = {0};
   int device = 0;
   cudaGetDevice(&device);
   if (device >= 64 || S < 2 || S > 4) return 0;
-  if (!attr_done[device]) {
-    if (cudaFuncSetAttribute(gemm_tc_sk_kernel<BN, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             C::SMEM_BYTES) != cudaSuccess ||
-        cudaFuncSetAttribute(gemm_tc_sk_kernel<BN, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             C::SMEM_BYTES) != cudaSuccess)
-      return 0;
-    attr_done[device] = 1;
-  }
+  if (allow_smem<gemm_tc_sk_kernel<BN, false>, C::SMEM_BYTES>() != cudaSuccess ||
+      allow_smem<gemm_tc_sk_kernel<BN, true>, C::SMEM_BYTES>() != cudaSuccess)
+    return 0;
   if (!cache[device][S]) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(S * (dev.num_sms / S)));

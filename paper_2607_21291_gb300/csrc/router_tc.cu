@@ -506,12 +506,8 @@ cudaError_t router_tc(const void* x, int64_t rows, int d, const void* w1, const 
   if (!make_tmap_bf16(&tx, x, (uint64_t)rows, (uint64_t)d, (uint64_t)d, kRK, kRM) ||
       !make_tmap_bf16(&tw, w1, (uint64_t)kRN, (uint64_t)d, (uint64_t)d, kRK, kRN))
     return cudaErrorInvalidValue;
-  static std::once_flag attr_once;
-  static cudaError_t attr_err = cudaSuccess;
-  std::call_once(attr_once, [] {
-    attr_err = cudaFuncSetAttribute(router_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRSmem);
-  });
-  if (attr_err != cudaSuccess) return attr_err;
+  const cudaError_t e = allow_smem<router_tc_kernel, kRSmem>();
+  if (e != cudaSuccess) return e;
   return launch_pdl(router_tc_kernel, dim3(p.G), dim3(kRThreads), kRSmem, dev.stream, tx, tw, p);
 }
 

@@ -890,16 +890,8 @@ cudaError_t gather_norm_launch(const void* x, const int32_t* rows, int64_t M, in
                                void* out2, const Dev& dev) {
   const size_t row_bytes = (size_t)d * sizeof(T);
   const size_t smem = 4 * row_bytes + kRowSlots * row_bytes + 2 * kRowSlots * 8;
-  static int attr_done[64] = {0};
-  int device = 0;
-  cudaGetDevice(&device);
-  if (device < 64 && !attr_done[device]) {
-    cudaError_t e = cudaFuncSetAttribute(gather_norm_tma_kernel<T, RMS, NCH>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (4 + kRowSlots) * kMaxRowBytes + 2 * kRowSlots * 8);
-    if (e != cudaSuccess) return e;
-    attr_done[device] = 1;
-  }
+  const cudaError_t e = allow_smem<gather_norm_tma_kernel<T, RMS, NCH>, (4 + kRowSlots) * kMaxRowBytes + 2 * kRowSlots * 8>();
+  if (e != cudaSuccess) return e;
   // one wave: as many blocks per SM as fit (at most two), at least one row
   // per consumer warp
   const int64_t fit = std::max<int64_t>(1, std::min<int64_t>(2, 232448 / (int64_t)(smem + 1024)));
@@ -1034,15 +1026,8 @@ cudaError_t topk(const float* scores, int B, int T, int K, int32_t* idx, int32_t
                  const Dev& dev) {
   if (B <= 0 || K <= 0) return cudaSuccess;
   const size_t smem = (size_t)T * sizeof(uint32_t);
-  static int attr_done[64] = {0};
-  int device = 0;
-  cudaGetDevice(&device);
-  if (device < 64 && !attr_done[device]) {
-    cudaError_t e = cudaFuncSetAttribute(topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         kMaxTopkT * (int)sizeof(uint32_t));
-    if (e != cudaSuccess) return e;
-    attr_done[device] = 1;
-  }
+  const cudaError_t e = allow_smem<topk_kernel, kMaxTopkT * (int)sizeof(uint32_t)>();
+  if (e != cudaSuccess) return e;
   return launch_pdl(topk_kernel, dim3(B), dim3(kTopkThreads), smem, dev.stream, scores, T, K, idx,
                     rows);
 }
@@ -1063,15 +1048,8 @@ cudaError_t select_gather_norm_t(const float* scores, int B, int seq_len, int K,
   const int G = (int)std::max<int64_t>(1, (K + per_block - 1) / per_block);
   return with_nch<T>(d, [&](auto nch) -> cudaError_t {
     constexpr int NCH = decltype(nch)::value;
-    static int attr_done[64] = {0};
-    int device = 0;
-    cudaGetDevice(&device);
-    if (device < 64 && !attr_done[device]) {
-      cudaError_t e = cudaFuncSetAttribute(select_gather_norm_kernel<T, RMS, NCH>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, kSelSmemMax);
-      if (e != cudaSuccess) return e;
-      attr_done[device] = 1;
-    }
+    const cudaError_t e = allow_smem<select_gather_norm_kernel<T, RMS, NCH>, kSelSmemMax>();
+    if (e != cudaSuccess) return e;
     return launch_pdl(select_gather_norm_kernel<T, RMS, NCH>, dim3(G, B), dim3(kSelThreads), smem,
                       dev.stream, scores, seq_len, K, static_cast<const T*>(x), d,
                       static_cast<const T*>(g1), static_cast<const T*>(b1),

@@ -36,3 +36,16 @@ def test_erf_fit_matches_kernel_and_bound():
     assert np.allclose(kern, c, rtol=1e-6, atol=0)
     z = np.linspace(0, 8, 200001)
     assert np.max(np.abs(m.erf_fp32(z, c).astype(np.float64) - erf(z))) <= 3.3e-7
+
+
+def test_shared_memory_limits_are_constants():
+    """A kernel's shared-memory limit belongs to the function and the device: one
+    helper sets it, to a compile-time constant, so that no call can lower it for
+    another host thread's launch."""
+    places = []
+    for f in sorted(os.listdir(CSRC)):
+        if f.endswith((".cu", ".cuh", ".h")):
+            src = open(os.path.join(CSRC, f)).read()
+            places += [(f, src[max(0, m.start() - 400):m.end() + 120]) for m in re.finditer("cudaFuncSetAttribute", src)]
+    assert [f for f, _ in places] == ["common.cuh"]
+    assert "allow_smem()" in places[0][1] and "MaxDynamicSharedMemorySize, BYTES)" in places[0][1]
