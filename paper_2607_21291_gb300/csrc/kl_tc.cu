@@ -9,7 +9,7 @@
 // Storing the logits and reading them back cost more than the products: 4 bytes
 // written and three times read per class, row and model (2 GB at 1000 rows of
 // 50304 classes). There the whole loss took 1492 us (two projections of 123 us
-// and a pass of 964 us over the logits); it takes 121 us here, bound by the rate
+// and a pass of 964 us over the logits); it takes 126 us here, bound by the rate
 // at which one thread issues N = 128 products (two a 16-deep k step); W comes
 // from HBM once, since the row blocks walk the classes side by side.
 //
